@@ -59,8 +59,8 @@ mdf_status mdf_net_set_stream(mdf_net *net, void *cuda_stream);
  * the resolution of the layer is a power of two, and on the mma.sync kernel
  * otherwise; kind 1 runs every convolution on the mma.sync kernel (the
  * reference point the tcgen05 kernel is measured and tested against).  The
- * weight gradient runs on the mma.sync kernel.  MDF_E_INVALID for another
- * kind. */
+ * weight gradient follows the same choice (tcgen05 from 8 x 8 upwards).
+ * MDF_E_INVALID for another kind. */
 mdf_status mdf_net_set_conv_kernel(mdf_net *net, int kind);
 
 /* Number of parameters; layer count and the real (cout, cin) of a layer. */

@@ -175,7 +175,8 @@ static mdf_status wgrad(mdf_net *n, int l, int B, const bf16 *dZ, const bf16 *X)
     a.Cout = n->cout_pad[l];
     a.cin_real = kLayers[l].cin;
     a.cout_real = kLayers[l].cout;
-    NCK(n, conv_wgrad(a, n->num_sms, n->stream));
+    if (n->conv_kind == 0 && conv_wgrad_tc_applies(a)) NCK(n, conv_wgrad_tc(a, n->num_sms, n->err, n->stream));
+    else NCK(n, conv_wgrad(a, n->num_sms, n->stream));
     return MDF_OK;
 }
 

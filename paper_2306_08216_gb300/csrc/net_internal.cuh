@@ -65,6 +65,11 @@ struct WGradArgs {
     int B, R, Cin, Cout, cin_real, cout_real;
 };
 cudaError_t conv_wgrad(const WGradArgs &a, int num_sms, cudaStream_t st);
+// The same sums on the tcgen05 tensor cores (net_wgrad.cu).  Applies when R is
+// a power of two of at least 8, Cin is 32 or a multiple of 64 and Cout 32, 64
+// or a multiple of 128; a CTA that gives up waiting sets *err (device memory).
+bool conv_wgrad_tc_applies(const WGradArgs &a);
+cudaError_t conv_wgrad_tc(const WGradArgs &a, int num_sms, int *err, cudaStream_t st);
 
 // Elementwise / layout kernels (n = element count unless stated).
 cudaError_t silu_forward(const bf16 *z, bf16 *y, long long n, cudaStream_t st);

@@ -6,7 +6,9 @@
 // one filter tap per 32-wide K step straight from the NHWC activations (zero
 // outside the image) into double-buffered shared memory.  The weight
 // gradient is the transposed product, split over pixels and reduced with
-// FP32 atomics into the flat gradient vector.
+// FP32 atomics into the flat gradient vector.  Both serve the sides that the
+// tcgen05 kernels (net_tc.cu, net_wgrad.cu) do not, and are what those are
+// tested against.
 #include <math.h>
 
 #include "net_internal.cuh"
@@ -211,13 +213,21 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WGradArgs a, int chunk) {
         }
     };
 
-    float acc[2][4][4];
+    // The MMAs' FP32 accumulation drops low bits at every step: chains of at
+    // most 16 of them (8 K tiles), with rounded additions in between.
+    float acc[2][4][4], sum[2][4][4];
+    auto flush = [&](bool first) {
 #pragma unroll
-    for (int mi = 0; mi < 2; ++mi)
+        for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
-        for (int ni = 0; ni < 4; ++ni)
+            for (int ni = 0; ni < 4; ++ni)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[mi][ni][e] = 0.0f;
+                for (int e = 0; e < 4; ++e) {
+                    sum[mi][ni][e] = first ? 0.0f : sum[mi][ni][e] + acc[mi][ni][e];
+                    acc[mi][ni][e] = 0.0f;
+                }
+    };
+    flush(true);
 
     load(kt0);
     store(0);
@@ -227,8 +237,10 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WGradArgs a, int chunk) {
         if (kt + 1 < kt1) load(kt + 1);
         warp_tile_k32(As[cur], Bs[cur], wm * 32, wn * 32, lane, acc);
         if (kt + 1 < kt1) store(cur ^ 1);
+        if (((kt - kt0) & 7) == 7) flush(false);
         __syncthreads();
     }
+    flush(false);
 
     const int g = lane >> 2, c = lane & 3;
 #pragma unroll
@@ -242,7 +254,7 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WGradArgs a, int chunk) {
                 if (co >= a.cout_real || n >= NC) continue;
                 const int tap = n / a.Cin, ci = n - tap * a.Cin;
                 if (ci >= a.cin_real) continue;
-                atomicAdd(a.g + a.off + ((long long)co * 9 + tap) * a.cin_real + ci, acc[mi][ni][e]);
+                atomicAdd(a.g + a.off + ((long long)co * 9 + tap) * a.cin_real + ci, sum[mi][ni][e]);
             }
 }
 

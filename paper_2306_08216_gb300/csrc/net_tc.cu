@@ -27,136 +27,16 @@
 // Every wait is bounded (about two seconds).  A CTA that gives up records
 // an error word, waits (bounded) for its own copies and MMAs to finish,
 // frees its TMEM and returns; the host reports the word as MDF_E_CUDA.
-#include <cuda.h>
-#include <cudaTypedefs.h>
-
-#include <atomic>
-
-#include "net_internal.cuh"
+#include "net_tc.cuh"
 
 namespace mdfnet {
 
 namespace {
 
-constexpr int TC_BM = 128;
 // warp 0: TMA, warp 1: MMA, warps 2-9: epilogue (two warps per TMEM lane
 // quarter, each taking half of the accumulator's columns)
 constexpr int TC_EPI_WARPS = 8;
 constexpr int TC_THREADS = 32 * (2 + TC_EPI_WARPS);
-
-__device__ __forceinline__ uint32_t s_u32(const void *p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mb_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mb_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbarrier_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mb_try_wait(uint64_t *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(s_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait: gives up after ~2^32 clock cycles (about two seconds).
-__device__ __forceinline__ bool mb_wait(uint64_t *bar, uint32_t parity) {
-    if (mb_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (true) {
-        if (mb_try_wait(bar, parity)) return true;
-        if (clock64() - t0 > (1ll << 32)) return false;
-    }
-}
-
-__device__ __forceinline__ void tma_load_4d(const CUtensorMap *map, uint64_t *bar, void *dst, int c0, int c1, int c2,
-                                            int c3) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
-        "[%6];" ::"r"(s_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(s_u32(bar))
-        : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(const CUtensorMap *map, uint64_t *bar, void *dst, int c0, int c1,
-                                            int c2) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
-            "r"(s_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(s_u32(bar))
-        : "memory");
-}
-
-// ---- tcgen05 (tensor memory and the fifth-generation MMA)
-
-__device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s_u32(dst_smem)),
-                 "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// D[tmem] (+)= A[smem] x B[smem]^T, one M = 128, N = BN, K = 16 step.
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// Arrive on `bar` once every MMA this thread issued before has completed.
-__device__ __forceinline__ void umma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s_u32(bar))
-                 : "memory");
-}
-// 16 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// Shared-memory matrix descriptor of a K-major operand in the swizzled
-// layout TMA writes: rows of BKC x 2 bytes, 8-row groups SBO bytes apart;
-// start address and offsets in 16-byte units, version 1 (bits 46-47),
-// swizzle mode in bits 61-63 (2: 128-byte, 4: 64-byte).
-template <int BKC>
-__device__ __forceinline__ uint64_t kmajor_desc(uint32_t saddr) {
-    constexpr uint64_t sbo = 8 * BKC * 2;         // bytes between 8-row groups
-    constexpr uint64_t layout = BKC == 64 ? 2 : 4;
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((sbo >> 4) << 32) | ((uint64_t)1 << 46) |
-           (layout << 61);
-}
-
-// Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), BF16
-// A and B (bits 7-9 = 1, 10-12 = 1), both K-major (bits 15, 16 = 0),
-// N >> 3 in bits 17-22, M >> 4 in bits 24-28.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
 
 struct TcTile {
     int Wx, Hy, Bn;  // the 128-pixel tile as columns x rows x images
@@ -176,18 +56,6 @@ struct TcSmem {
     static constexpr int NBAR = 2 * STAGES + 5;
     static constexpr int TOTAL = BARS + NBAR * 8 + 16 + 1024;  // + alignment slack
 };
-
-// Bounded wait that also gives up as soon as another role of the CTA has
-// failed (*fail set).
-__device__ __forceinline__ bool mb_wait_f(uint64_t *bar, uint32_t parity, volatile int *fail) {
-    if (mb_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (true) {
-        if (mb_try_wait(bar, parity)) return true;
-        if (*fail) return false;
-        if (clock64() - t0 > (1ll << 32)) return false;
-    }
-}
 
 // Persistent, warp-specialised CTA of TC_THREADS threads walking output tiles
 // tile = blockIdx.x, blockIdx.x + gridDim.x, ... (tile = m_tile * ntn + n_tile):
@@ -412,22 +280,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 }
 
 // ---- host side
-
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-    static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> fn{nullptr};
-    PFN_cuTensorMapEncodeTiled_v12000 f = fn.load();
-    if (!f) {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess || !p)
-            return nullptr;
-        f = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-        fn.store(f);
-    }
-    return f;
-}
 
 // The tile shape for side R: P pixels (a power of two) as whole rows of
 // whole images when R <= P, a P-column piece of one row otherwise (each box
