@@ -54,13 +54,14 @@ struct mdf_net {
     bf16 *p0 = nullptr, *p1 = nullptr, *p2 = nullptr, *u0 = nullptr, *u1 = nullptr, *u2 = nullptr;
     float *outf = nullptr, *tgt = nullptr, *io = nullptr;
     // gradients
-    bf16 *dz[kNL], *dy[kNL];
+    bf16 *dz[kNL];
     bf16 *dp0 = nullptr, *dp1 = nullptr, *dp2 = nullptr, *du0 = nullptr, *du1 = nullptr, *du2 = nullptr;
     double *loss = nullptr, *h_loss = nullptr;
     int *err = nullptr, *h_err = nullptr;  // error word of the tensor-core kernels
     int conv_kind = 0;                     // 0: tcgen05 where it applies, 1: mma.sync
     long long adam_t = 0;
     bool prepared = false;
+    bool keep_z = true;                    // the forward pass at hand precedes a backward pass
     char last_error[256] = {0};
 };
 
@@ -112,9 +113,23 @@ static long long pix(const mdf_net *n, int B, int div) {
 
 // Rebuild the BF16 layer weights from the FP32 master parameters.
 static mdf_status prepare(mdf_net *n) {
-    for (int l = 0; l < kNL; ++l)
-        NCK(n, prepare_layer(n->params, n->off[l], kLayers[l].cin, kLayers[l].cout, n->cin_pad[l], n->cout_pad[l],
-                             n->wf[l], n->wb[l], n->bias[l], n->stream));
+    static_assert(kNL <= kMaxLayers, "layer table");
+    PrepareArgs a;
+    a.params = n->params;
+    a.layers = kNL;
+    a.first[0] = 0;
+    for (int l = 0; l < kNL; ++l) {
+        a.first[l + 1] = a.first[l] + (long long)n->cout_pad[l] * 9 * n->cin_pad[l];
+        a.off[l] = n->off[l];
+        a.cin_real[l] = kLayers[l].cin;
+        a.cout_real[l] = kLayers[l].cout;
+        a.cin_pad[l] = n->cin_pad[l];
+        a.cout_pad[l] = n->cout_pad[l];
+        a.wf[l] = n->wf[l];
+        a.wb[l] = n->wb[l];
+        a.bias[l] = n->bias[l];
+    }
+    NCK(n, prepare_layers(a, n->stream));
     n->prepared = true;
     return MDF_OK;
 }
@@ -136,6 +151,7 @@ static mdf_status conv(mdf_net *n, int l, int B, const bf16 *x, const bf16 *skip
     a.skip = skip;
     a.out = out;
     a.act = act;
+    a.zgrad = nullptr;
     a.outf = outf;
     a.nf = nf;
     a.B = B;
@@ -145,8 +161,9 @@ static mdf_status conv(mdf_net *n, int l, int B, const bf16 *x, const bf16 *skip
     return run_conv(n, a);
 }
 
-// dX of layer l's input from dZ (mirrored weights, no bias).
-static mdf_status conv_dx(mdf_net *n, int l, int B, const bf16 *dZ, bf16 *dX) {
+// dX of layer l's input from dZ (mirrored weights, no bias), times silu'(z)
+// where the input is the activation of z.
+static mdf_status conv_dx(mdf_net *n, int l, int B, const bf16 *dZ, bf16 *dX, const bf16 *z = nullptr) {
     ConvArgs a;
     a.X = dZ;
     a.W = n->wb[l];
@@ -154,6 +171,7 @@ static mdf_status conv_dx(mdf_net *n, int l, int B, const bf16 *dZ, bf16 *dX) {
     a.skip = nullptr;
     a.out = dX;
     a.act = nullptr;
+    a.zgrad = z;
     a.outf = nullptr;
     a.nf = 0;
     a.B = B;
@@ -187,9 +205,10 @@ static mdf_status wgrad(mdf_net *n, int l, int B, const bf16 *dZ, const bf16 *X)
     } while (0)
 
 // Layer l with its activation: z = conv(x) + b (+ skip), y = silu(z), the
-// activation written by the convolution's epilogue.
+// activation written by the convolution's epilogue; z only where a backward
+// pass will read it.
 static mdf_status layer(mdf_net *n, int l, int B, const bf16 *x, const bf16 *skip) {
-    return conv(n, l, B, x, skip, n->z[l], nullptr, 0, n->y[l]);
+    return conv(n, l, B, x, skip, n->keep_z ? n->z[l] : nullptr, nullptr, 0, n->y[l]);
 }
 
 static mdf_status forward(mdf_net *n, int B) {
@@ -218,10 +237,9 @@ static mdf_status forward(mdf_net *n, int B) {
     return conv(n, 14, B, n->y[13], nullptr, nullptr, n->outf, 3);
 }
 
-// dz[l] = silu'(z[l]) dy[l]
-static mdf_status act_back(mdf_net *n, int l, int B) {
-    NCK(n, silu_backward(n->z[l], n->dy[l], n->dz[l], pix(n, B, kLayers[l].div) * n->cout_pad[l], n->stream));
-    return MDF_OK;
+// dz of layer l - 1 from dz of layer l, whose input is its activation.
+static mdf_status back(mdf_net *n, int l, int B) {
+    return conv_dx(n, l, B, n->dz[l], n->dz[l - 1], n->z[l - 1]);
 }
 
 // Backward pass from dz[14] (dLoss/dout, set by the loss kernel) into grad.
@@ -230,62 +248,45 @@ static mdf_status backward(mdf_net *n, int B) {
     NCK(n, cudaMemsetAsync(n->grad, 0, n->P * sizeof(float), n->stream));
     // output layer and the R-level decoder
     NRET(wgrad(n, 14, B, n->dz[14], n->y[13]));
-    NRET(conv_dx(n, 14, B, n->dz[14], n->dy[13]));
-    NRET(act_back(n, 13, B));
+    NRET(back(n, 14, B));
     NRET(wgrad(n, 13, B, n->dz[13], n->y[12]));
-    NRET(conv_dx(n, 13, B, n->dz[13], n->dy[12]));
-    NRET(act_back(n, 12, B));
+    NRET(back(n, 13, B));
     NRET(wgrad(n, 12, B, n->dz[12], n->u0));
     NRET(conv_dx(n, 12, B, n->dz[12], n->du0));
-    NCK(n, up_backward(n->du0, n->dy[11], B, R / 2, 64, n->stream));
+    NCK(n, up_backward(n->du0, n->z[11], n->dz[11], B, R / 2, 64, n->stream));
     // R/2 decoder
-    NRET(act_back(n, 11, B));
     NRET(wgrad(n, 11, B, n->dz[11], n->y[10]));
-    NRET(conv_dx(n, 11, B, n->dz[11], n->dy[10]));
-    NRET(act_back(n, 10, B));
+    NRET(back(n, 11, B));
     NRET(wgrad(n, 10, B, n->dz[10], n->u1));
     NRET(conv_dx(n, 10, B, n->dz[10], n->du1));
-    NCK(n, up_backward(n->du1, n->dy[9], B, R / 4, 128, n->stream));
+    NCK(n, up_backward(n->du1, n->z[9], n->dz[9], B, R / 4, 128, n->stream));
     // R/4 decoder
-    NRET(act_back(n, 9, B));
     NRET(wgrad(n, 9, B, n->dz[9], n->y[8]));
-    NRET(conv_dx(n, 9, B, n->dz[9], n->dy[8]));
-    NRET(act_back(n, 8, B));
+    NRET(back(n, 9, B));
     NRET(wgrad(n, 8, B, n->dz[8], n->u2));
     NRET(conv_dx(n, 8, B, n->dz[8], n->du2));
-    NCK(n, up_backward(n->du2, n->dy[7], B, R / 8, 256, n->stream));
+    NCK(n, up_backward(n->du2, n->z[7], n->dz[7], B, R / 8, 256, n->stream));
     // bottleneck
-    NRET(act_back(n, 7, B));
     NRET(wgrad(n, 7, B, n->dz[7], n->y[6]));
-    NRET(conv_dx(n, 7, B, n->dz[7], n->dy[6]));
-    NRET(act_back(n, 6, B));
+    NRET(back(n, 7, B));
     NRET(wgrad(n, 6, B, n->dz[6], n->p2));
     NRET(conv_dx(n, 6, B, n->dz[6], n->dp2));
     // encoder R/4: s2 receives the pooled path and the skip of d2a
-    NCK(n, pool_backward(n->dp2, n->dy[5], B, R / 4, 128, n->stream));
-    NCK(n, add_inplace(n->dy[5], n->dz[8], pix(n, B, 4) * 128, n->stream));
-    NRET(act_back(n, 5, B));
+    NCK(n, pool_backward(n->dp2, n->dz[8], n->z[5], n->dz[5], B, R / 4, 128, n->stream));
     NRET(wgrad(n, 5, B, n->dz[5], n->y[4]));
-    NRET(conv_dx(n, 5, B, n->dz[5], n->dy[4]));
-    NRET(act_back(n, 4, B));
+    NRET(back(n, 5, B));
     NRET(wgrad(n, 4, B, n->dz[4], n->p1));
     NRET(conv_dx(n, 4, B, n->dz[4], n->dp1));
     // encoder R/2
-    NCK(n, pool_backward(n->dp1, n->dy[3], B, R / 2, 64, n->stream));
-    NCK(n, add_inplace(n->dy[3], n->dz[10], pix(n, B, 2) * 64, n->stream));
-    NRET(act_back(n, 3, B));
+    NCK(n, pool_backward(n->dp1, n->dz[10], n->z[3], n->dz[3], B, R / 2, 64, n->stream));
     NRET(wgrad(n, 3, B, n->dz[3], n->y[2]));
-    NRET(conv_dx(n, 3, B, n->dz[3], n->dy[2]));
-    NRET(act_back(n, 2, B));
+    NRET(back(n, 3, B));
     NRET(wgrad(n, 2, B, n->dz[2], n->p0));
     NRET(conv_dx(n, 2, B, n->dz[2], n->dp0));
     // encoder R
-    NCK(n, pool_backward(n->dp0, n->dy[1], B, R, 32, n->stream));
-    NCK(n, add_inplace(n->dy[1], n->dz[12], pix(n, B, 1) * 32, n->stream));
-    NRET(act_back(n, 1, B));
+    NCK(n, pool_backward(n->dp0, n->dz[12], n->z[1], n->dz[1], B, R, 32, n->stream));
     NRET(wgrad(n, 1, B, n->dz[1], n->y[0]));
-    NRET(conv_dx(n, 1, B, n->dz[1], n->dy[0]));
-    NRET(act_back(n, 0, B));
+    NRET(back(n, 1, B));
     return wgrad(n, 0, B, n->dz[0], n->xin);
 }
 
@@ -377,14 +378,12 @@ mdf_status mdf_net_create(int resolution, int max_batch, mdf_net **out) {
         const size_t act = (size_t)pix(n, B, kLayers[l].div) * n->cout_pad[l];
         NCKC(nalloc(n, &n->z[l], act));
         NCKC(nalloc(n, &n->dz[l], act));
-        n->y[l] = n->dy[l] = nullptr;
-        if (kLayers[l].act) {
-            NCKC(nalloc(n, &n->y[l], act));
-            NCKC(nalloc(n, &n->dy[l], act));
-        }
+        n->y[l] = nullptr;
+        if (kLayers[l].act) NCKC(nalloc(n, &n->y[l], act));
     }
     const int R = resolution;
     NCKC(nalloc(n, &n->xin, (size_t)pix(n, B, 1) * 32));
+    NCKE(cudaMemset(n->xin, 0, (size_t)pix(n, B, 1) * 32 * sizeof(bf16)));  // channels past the input planes stay zero
     NCKC(nalloc(n, &n->p0, (size_t)pix(n, B, 2) * 32));
     NCKC(nalloc(n, &n->p1, (size_t)pix(n, B, 4) * 64));
     NCKC(nalloc(n, &n->p2, (size_t)pix(n, B, 8) * 128));
@@ -406,6 +405,7 @@ mdf_status mdf_net_create(int resolution, int max_batch, mdf_net **out) {
     NCKE(cudaMemset(n->err, 0, sizeof(int)));
     NCKE(cudaMallocHost(&n->h_err, sizeof(int)));
     *n->h_err = 0;
+    NCKE(cudaStreamSynchronize(nullptr));  // the cleared buffers, before any other stream uses them
     (void)R;
     *out = n;
     return MDF_OK;
@@ -464,6 +464,7 @@ mdf_status mdf_net_forward(mdf_net *n, int batch, const float *inputs, float *ou
     if (!n) return MDF_E_INVALID;
     NRET(check_batch(n, batch, inputs, outputs));
     NRET(stage(n, batch, inputs, nullptr, on_device));
+    n->keep_z = false;
     NRET(forward(n, batch));
     const long long RR = (long long)n->R * n->R;
     float *dst = on_device ? outputs : n->io;
@@ -477,6 +478,7 @@ mdf_status mdf_net_forward(mdf_net *n, int batch, const float *inputs, float *ou
 static mdf_status loss_and_backward(mdf_net *n, int batch, const float *inputs, const float *targets,
                                     int on_device) {
     NRET(stage(n, batch, inputs, targets, on_device));
+    n->keep_z = true;
     NRET(forward(n, batch));
     NCK(n, mse_loss(n->outf, n->tgt, n->dz[14], n->loss, batch, n->R, n->stream));
     return backward(n, batch);

@@ -30,6 +30,14 @@ __device__ __forceinline__ __nv_bfloat16 silu_bf16(__nv_bfloat16 zb) {
     return __float2bfloat16_rn(v * net_sigmoid(v));
 }
 
+// dz = dy silu'(z) of BF16 values, silu'(z) = s (1 + z (1 - s)), s =
+// sigmoid(z), rounded to BF16 by the caller: shared by the elementwise kernels
+// and the convolution epilogues that fuse it.
+__device__ __forceinline__ float silu_grad(float dy, float z) {
+    const float sg = net_sigmoid(z);
+    return dy * sg * (1.0f + z * (1.0f - sg));
+}
+
 // out[m][n] = sum_k A[m][k] W[n][k] (+ bias[n]) (+ skip[m][n]) over
 // k = (tap, c), A[m][(tap, c)] = X[pixel m shifted by tap][c] (zero outside):
 // the forward convolution (X = activations, W = [Cout][9][Cin]) and the input
@@ -39,8 +47,9 @@ struct ConvArgs {
     const bf16 *W;      // [N][9][Cx]
     const float *bias;  // [N] or null
     const bf16 *skip;   // [B][R][R][N] or null
-    bf16 *out;          // [B][R][R][N] (N % 2 == 0), or null if outf is set
+    bf16 *out;          // [B][R][R][N] (N % 2 == 0), or null
     bf16 *act;          // SiLU of the BF16-rounded out, [B][R][R][N], or null
+    const bf16 *zgrad;  // out = BF16-rounded sum times silu'(zgrad), [B][R][R][N], or null
     float *outf;        // FP32 output [B][R][R][nf] of the first nf channels, or null
     int nf;
     int B, R, Cx, N;
@@ -73,14 +82,18 @@ cudaError_t conv_wgrad_tc(const WGradArgs &a, int num_sms, int *err, cudaStream_
 
 // Elementwise / layout kernels (n = element count unless stated).
 cudaError_t silu_forward(const bf16 *z, bf16 *y, long long n, cudaStream_t st);
-cudaError_t silu_backward(const bf16 *z, const bf16 *dy, bf16 *dz, long long n, cudaStream_t st);
 cudaError_t pool_forward(const bf16 *x, bf16 *y, int B, int R, int C, cudaStream_t st);    // R = input side
-cudaError_t pool_backward(const bf16 *dy, bf16 *dx, int B, int R, int C, cudaStream_t st); // dx = ...
+// dz [B][R][R][C] = silu'(z) (dy [B][R/2][R/2][C] / 4 + skip), the gradient
+// through a pooled activation that also feeds a skip connection; the quarter
+// and the sum are rounded to BF16
+cudaError_t pool_backward(const bf16 *dy, const bf16 *skip, const bf16 *z, bf16 *dz, int B, int R, int C,
+                          cudaStream_t st);
 cudaError_t up_forward(const bf16 *x, bf16 *y, int B, int R, int C, cudaStream_t st);      // R = input side
-cudaError_t up_backward(const bf16 *dy, bf16 *dx, int B, int R, int C, cudaStream_t st);
-cudaError_t add_inplace(bf16 *dst, const bf16 *src, long long n, cudaStream_t st);
-// planar FP32 [B][NET_IN_PLANES][R][R] -> NHWC BF16 [B][R][R][32] (zero
-// channels NET_IN_PLANES..31)
+// dz [B][R][R][C] = silu'(z) times the (BF16-rounded) sum of the four children
+// of dy [B][2R][2R][C]
+cudaError_t up_backward(const bf16 *dy, const bf16 *z, bf16 *dz, int B, int R, int C, cudaStream_t st);
+// planar FP32 [B][NET_IN_PLANES][R][R] -> channels 0..NET_IN_PLANES-1 of NHWC
+// BF16 [B][R][R][32] (the caller cleared the others once)
 cudaError_t pack_input(const float *in, bf16 *x, int B, int R, cudaStream_t st);
 // NHWC FP32 [B][R][R][3] <-> planar FP32 [B][3][R][R]
 cudaError_t unpack_output(const float *o, float *out, int B, int R, cudaStream_t st);
@@ -89,10 +102,19 @@ cudaError_t pack_target(const float *t, float *o, int B, int R, cudaStream_t st)
 // dOut = 2 (o - t) / count as NHWC BF16 [B][R][R][32] (zero channels 3..31)
 cudaError_t mse_loss(const float *o, const float *t, bf16 *dout, double *loss, int B, int R, cudaStream_t st);
 // Layer weights from the flat FP32 parameter vector: forward BF16
-// [cout_pad][9][cin_pad], mirrored BF16 [cin_pad][9][cout_pad] (may be null)
-// and FP32 bias [cout_pad], zero in the padding.
-cudaError_t prepare_layer(const float *params, long long off, int cin_real, int cout_real, int cin_pad,
-                          int cout_pad, bf16 *wf, bf16 *wb, float *bias, cudaStream_t st);
+// [cout_pad][9][cin_pad], mirrored BF16 [cin_pad][9][cout_pad] and FP32 bias
+// [cout_pad], zero in the padding; every layer in one launch.
+constexpr int kMaxLayers = 16;
+struct PrepareArgs {
+    const float *params;
+    int layers;
+    long long first[kMaxLayers + 1];  // first work item of each layer, then their number
+    long long off[kMaxLayers];
+    int cin_real[kMaxLayers], cout_real[kMaxLayers], cin_pad[kMaxLayers], cout_pad[kMaxLayers];
+    bf16 *wf[kMaxLayers], *wb[kMaxLayers];
+    float *bias[kMaxLayers];
+};
+cudaError_t prepare_layers(const PrepareArgs &a, cudaStream_t st);
 // Adam on the flat vector: m = b1 m + (1 - b1) g, v = b2 v + (1 - b2) g^2,
 // p -= lr_t m / (sqrt(v) + eps_t) with the bias-corrected step folded into
 // lr_t and eps_t.

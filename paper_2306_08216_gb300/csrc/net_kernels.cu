@@ -150,7 +150,13 @@ __global__ void __launch_bounds__(256) conv_kernel(ConvArgs a) {
                     v0 += s.x;
                     v1 += s.y;
                 }
-                const __nv_bfloat162 zb = __floats2bfloat162_rn(v0, v1);
+                __nv_bfloat162 zb = __floats2bfloat162_rn(v0, v1);
+                if (a.zgrad) {
+                    const float2 d = __bfloat1622float2(zb);
+                    const float2 z = __bfloat1622float2(
+                        *reinterpret_cast<const __nv_bfloat162 *>(a.zgrad + m * a.N + col));
+                    zb = __floats2bfloat162_rn(silu_grad(d.x, z.x), silu_grad(d.y, z.y));
+                }
                 if (a.out) *reinterpret_cast<__nv_bfloat162 *>(a.out + m * a.N + col) = zb;
                 if (a.act)
                     *reinterpret_cast<__nv_bfloat162 *>(a.act + m * a.N + col) =
@@ -271,8 +277,6 @@ __global__ void bias_grad_kernel(const bf16 *dZ, long long P, int Cout, int cout
 
 // ------------------------------------------------------------- elementwise
 
-__device__ __forceinline__ float sigm(float z) { return net_sigmoid(z); }
-
 __global__ void silu_fwd_kernel(const bf16 *z, bf16 *y, long long n) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         y[i] = silu_bf16(z[i]);
@@ -299,20 +303,7 @@ __device__ __forceinline__ bf16x8 pack8(const float f[8]) {
     return w;
 }
 
-// dz = dy silu'(z), silu'(z) = s (1 + z (1 - s)), s = sigmoid(z); n8 = n / 8
-__global__ void silu_bwd_kernel(const bf16x8 *z, const bf16x8 *dy, bf16x8 *dz, long long n8) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += (long long)gridDim.x * blockDim.x) {
-        float a[8], b[8];
-        unpack8(z[i], a);
-        unpack8(dy[i], b);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const float sg = sigm(a[e]);
-            b[e] = b[e] * sg * (1.0f + a[e] * (1.0f - sg));
-        }
-        dz[i] = pack8(b);
-    }
-}
+__device__ __forceinline__ float round_bf16(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
 // x [B][R][R][C] -> y [B][R/2][R/2][C]; C8 = C / 8
 __global__ void pool_fwd_kernel(const bf16x8 *x, bf16x8 *y, int B, int R, int C8) {
@@ -337,8 +328,9 @@ __global__ void pool_fwd_kernel(const bf16x8 *x, bf16x8 *y, int B, int R, int C8
     }
 }
 
-// dy [B][R/2][R/2][C] -> dx [B][R][R][C] = dy / 4 on each 2 x 2 block
-__global__ void pool_bwd_kernel(const bf16x8 *dy, bf16x8 *dx, int B, int R, int C8) {
+// dy [B][R/2][R/2][C], skip, z [B][R][R][C] -> dz = silu'(z) (dy / 4 + skip)
+__global__ void pool_bwd_kernel(const bf16x8 *dy, const bf16x8 *skip, const bf16x8 *z, bf16x8 *dz, int B, int R,
+                                int C8) {
     const long long n = (long long)B * R * R * C8;
     const int h = R / 2;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -348,11 +340,15 @@ __global__ void pool_bwd_kernel(const bf16x8 *dy, bf16x8 *dx, int B, int R, int 
         t /= R;
         const int y = (int)(t % R);
         const long long b = t / R;
-        float f[8];
+        float f[8], g[8], a[8];
         unpack8(dy[((b * h + y / 2) * h + x / 2) * C8 + c], f);
+        unpack8(skip[i], g);
+        unpack8(z[i], a);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) f[e] *= 0.25f;
-        dx[i] = pack8(f);
+        for (int e = 0; e < 8; ++e) f[e] = round_bf16(round_bf16(f[e] * 0.25f) + g[e]);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) f[e] = silu_grad(f[e], a[e]);
+        dz[i] = pack8(f);
     }
 }
 
@@ -371,8 +367,8 @@ __global__ void up_fwd_kernel(const bf16x8 *x, bf16x8 *y, int B, int R, int C8) 
     }
 }
 
-// dy [B][2R][2R][C] -> dx [B][R][R][C] = sum of the four children
-__global__ void up_bwd_kernel(const bf16x8 *dy, bf16x8 *dx, int B, int R, int C8) {
+// dy [B][2R][2R][C], z [B][R][R][C] -> dz = silu'(z) times the sum of the four children
+__global__ void up_bwd_kernel(const bf16x8 *dy, const bf16x8 *z, bf16x8 *dz, int B, int R, int C8) {
     const int R2 = 2 * R;
     const long long n = (long long)B * R * R * C8;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -383,38 +379,32 @@ __global__ void up_bwd_kernel(const bf16x8 *dy, bf16x8 *dx, int B, int R, int C8
         const int y = (int)(t % R);
         const long long b = t / R;
         const long long base = ((b * R2 + 2 * y) * R2 + 2 * x) * C8 + c;
-        float p[8], q[8], r[8], u[8];
+        float p[8], q[8], r[8], u[8], a[8];
         unpack8(dy[base], p);
         unpack8(dy[base + C8], q);
         unpack8(dy[base + (long long)R2 * C8], r);
         unpack8(dy[base + (long long)R2 * C8 + C8], u);
+        unpack8(z[i], a);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) p[e] = p[e] + q[e] + r[e] + u[e];
-        dx[i] = pack8(p);
+        for (int e = 0; e < 8; ++e) p[e] = silu_grad(round_bf16(p[e] + q[e] + r[e] + u[e]), a[e]);
+        dz[i] = pack8(p);
     }
 }
 
-__global__ void add_kernel(bf16x8 *dst, const bf16x8 *src, long long n8) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += (long long)gridDim.x * blockDim.x) {
-        float a[8], b[8];
-        unpack8(dst[i], a);
-        unpack8(src[i], b);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) a[e] += b[e];
-        dst[i] = pack8(a);
-    }
-}
-
+// One 16-byte store per pixel: the eight planes as channels 0..7 (each plane
+// read coalesced); the other 24 channels stay zero from one call to the next.
+// 16 x 128^2: 54 us when every pixel's 32 channels were written one by one.
+static_assert(NET_IN_PLANES == 8, "one 16-byte group of channels per pixel");
 __global__ void pack_input_kernel(const float *in, bf16 *x, int B, int R) {
     const long long P = (long long)B * R * R;
     const int RR = R * R;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
         const long long b = p / RR;
         const int s = (int)(p - b * RR);
-        bf16 *o = x + p * 32;
+        float f[8];
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
-            o[c] = __float2bfloat16_rn(c < NET_IN_PLANES ? in[(b * NET_IN_PLANES + c) * RR + s] : 0.0f);
+        for (int c = 0; c < NET_IN_PLANES; ++c) f[c] = in[(b * NET_IN_PLANES + c) * RR + s];
+        *reinterpret_cast<bf16x8 *>(x + p * 32) = pack8(f);
     }
 }
 
@@ -461,19 +451,24 @@ __global__ void mse_kernel(const float *o, const float *t, bf16 *dout, double *l
     if ((threadIdx.x & 31) == 0) atomicAdd(loss, local * inv_count);
 }
 
-__global__ void prepare_kernel(const float *params, long long off, int cin_real, int cout_real, int cin_pad,
-                               int cout_pad, bf16 *wf, bf16 *wb, float *bias) {
-    const long long n = (long long)cout_pad * 9 * cin_pad;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+// Work item = one weight of one layer, consecutive in the forward layout.  One
+// launch for all layers: 15 of them took 71 us, mostly launch gaps.
+__global__ void prepare_kernel(const PrepareArgs a) {
+    const long long n = a.first[a.layers];
+    for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (long long)gridDim.x * blockDim.x) {
+        int l = 0;
+        while (g >= a.first[l + 1]) ++l;
+        const long long i = g - a.first[l];
+        const int cin_pad = a.cin_pad[l], cout_pad = a.cout_pad[l], cin_real = a.cin_real[l], cout_real = a.cout_real[l];
+        const float *p = a.params + a.off[l];
         const int ci = (int)(i % cin_pad);
-        const long long t = i / cin_pad;
-        const int tap = (int)(t % 9);
-        const int co = (int)(t / 9);
-        const float w = (co < cout_real && ci < cin_real) ? params[off + ((long long)co * 9 + tap) * cin_real + ci] : 0.0f;
+        const int t = (int)(i / cin_pad);
+        const int tap = t % 9, co = t / 9;
+        const float w = (co < cout_real && ci < cin_real) ? p[((long long)co * 9 + tap) * cin_real + ci] : 0.0f;
         const bf16 h = __float2bfloat16_rn(w);
-        wf[i] = h;
-        if (wb) wb[((long long)ci * 9 + (8 - tap)) * cout_pad + co] = h;
-        if (i < cout_pad) bias[i] = i < cout_real ? params[off + (long long)cout_real * 9 * cin_real + i] : 0.0f;
+        a.wf[l][i] = h;
+        a.wb[l][((long long)ci * 9 + (8 - tap)) * cout_pad + co] = h;
+        if (i < cout_pad) a.bias[l][i] = i < cout_real ? p[(long long)cout_real * 9 * cin_real + i] : 0.0f;
     }
 }
 
@@ -528,23 +523,18 @@ cudaError_t silu_forward(const bf16 *z, bf16 *y, long long n, cudaStream_t st) {
     silu_fwd_kernel<<<blocks_for(n), 256, 0, st>>>(z, y, n);
     return cudaGetLastError();
 }
-cudaError_t silu_backward(const bf16 *z, const bf16 *dy, bf16 *dz, long long n, cudaStream_t st) {
-    if (n % 8) return cudaErrorInvalidValue;
-    silu_bwd_kernel<<<blocks_for(n / 8), 256, 0, st>>>(reinterpret_cast<const bf16x8 *>(z),
-                                                      reinterpret_cast<const bf16x8 *>(dy),
-                                                      reinterpret_cast<bf16x8 *>(dz), n / 8);
-    return cudaGetLastError();
-}
 cudaError_t pool_forward(const bf16 *x, bf16 *y, int B, int R, int C, cudaStream_t st) {
     if (C % 8) return cudaErrorInvalidValue;
     pool_fwd_kernel<<<blocks_for((long long)B * R * R * C / 32), 256, 0, st>>>(
         reinterpret_cast<const bf16x8 *>(x), reinterpret_cast<bf16x8 *>(y), B, R, C / 8);
     return cudaGetLastError();
 }
-cudaError_t pool_backward(const bf16 *dy, bf16 *dx, int B, int R, int C, cudaStream_t st) {
+cudaError_t pool_backward(const bf16 *dy, const bf16 *skip, const bf16 *z, bf16 *dz, int B, int R, int C,
+                          cudaStream_t st) {
     if (C % 8) return cudaErrorInvalidValue;
     pool_bwd_kernel<<<blocks_for((long long)B * R * R * C / 8), 256, 0, st>>>(
-        reinterpret_cast<const bf16x8 *>(dy), reinterpret_cast<bf16x8 *>(dx), B, R, C / 8);
+        reinterpret_cast<const bf16x8 *>(dy), reinterpret_cast<const bf16x8 *>(skip),
+        reinterpret_cast<const bf16x8 *>(z), reinterpret_cast<bf16x8 *>(dz), B, R, C / 8);
     return cudaGetLastError();
 }
 cudaError_t up_forward(const bf16 *x, bf16 *y, int B, int R, int C, cudaStream_t st) {
@@ -553,16 +543,11 @@ cudaError_t up_forward(const bf16 *x, bf16 *y, int B, int R, int C, cudaStream_t
         reinterpret_cast<const bf16x8 *>(x), reinterpret_cast<bf16x8 *>(y), B, R, C / 8);
     return cudaGetLastError();
 }
-cudaError_t up_backward(const bf16 *dy, bf16 *dx, int B, int R, int C, cudaStream_t st) {
+cudaError_t up_backward(const bf16 *dy, const bf16 *z, bf16 *dz, int B, int R, int C, cudaStream_t st) {
     if (C % 8) return cudaErrorInvalidValue;
     up_bwd_kernel<<<blocks_for((long long)B * R * R * C / 8), 256, 0, st>>>(
-        reinterpret_cast<const bf16x8 *>(dy), reinterpret_cast<bf16x8 *>(dx), B, R, C / 8);
-    return cudaGetLastError();
-}
-cudaError_t add_inplace(bf16 *dst, const bf16 *src, long long n, cudaStream_t st) {
-    if (n % 8) return cudaErrorInvalidValue;
-    add_kernel<<<blocks_for(n / 8), 256, 0, st>>>(reinterpret_cast<bf16x8 *>(dst),
-                                                  reinterpret_cast<const bf16x8 *>(src), n / 8);
+        reinterpret_cast<const bf16x8 *>(dy), reinterpret_cast<const bf16x8 *>(z), reinterpret_cast<bf16x8 *>(dz), B, R,
+        C / 8);
     return cudaGetLastError();
 }
 cudaError_t pack_input(const float *in, bf16 *x, int B, int R, cudaStream_t st) {
@@ -584,10 +569,8 @@ cudaError_t mse_loss(const float *o, const float *t, bf16 *dout, double *loss, i
     mse_kernel<<<blocks_for(P), 256, 0, st>>>(o, t, dout, loss, P, 1.0 / (3.0 * (double)P));
     return cudaGetLastError();
 }
-cudaError_t prepare_layer(const float *params, long long off, int cin_real, int cout_real, int cin_pad,
-                          int cout_pad, bf16 *wf, bf16 *wb, float *bias, cudaStream_t st) {
-    prepare_kernel<<<blocks_for((long long)cout_pad * 9 * cin_pad), 256, 0, st>>>(params, off, cin_real, cout_real,
-                                                                                   cin_pad, cout_pad, wf, wb, bias);
+cudaError_t prepare_layers(const PrepareArgs &a, cudaStream_t st) {
+    prepare_kernel<<<blocks_for(a.first[a.layers]), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 cudaError_t adam_step(float *p, float *m, float *v, const float *g, long long n, float lr_t, float b1, float b2,

@@ -38,6 +38,22 @@ namespace {
 constexpr int TC_EPI_WARPS = 8;
 constexpr int TC_THREADS = 32 * (2 + TC_EPI_WARPS);
 
+// CTAs per SM and ring depth.  One thread issues a CTA's copies and one its
+// MMAs, and each ring slot costs them a few hundred cycles of issue and
+// barrier latency, so two CTAs per SM (two independent pipelines) run the
+// small layers about twice as fast as one CTA with a deeper ring, and a
+// slot carries as much work as its shared memory allows: two 32-channel K
+// steps (G = 2), or MT = 4 blocks of 128 pixels that share one weight box
+// (the 32-output-channel layers).  A ring takes about 104 KB of shared
+// memory per CTA (at most 16 slots); a CTA whose two accumulators fill
+// the 512 TMEM columns (BN = 256) runs alone on its SM with a 200 KB ring.
+constexpr int tc_ctas_per_sm(int acc_cols) { return 2 * acc_cols <= 256 ? 2 : 1; }
+constexpr int tc_stages(int stage, int acc_cols) {
+    return (tc_ctas_per_sm(acc_cols) == 2 ? 104 : 200) * 1024 / stage < 16
+               ? (tc_ctas_per_sm(acc_cols) == 2 ? 104 : 200) * 1024 / stage
+               : 16;
+}
+
 struct TcTile {
     int Wx, Hy, Bn;  // the 128-pixel tile as columns x rows x images
 };
@@ -69,8 +85,10 @@ struct TcSmem {
 //                    activation, BF16/FP32 stores, then release the
 //                    accumulator (tempty) so the MMAs of tile t + 2 may use it.
 // The epilogue of one tile overlaps the copies and MMAs of the next.
+// At most 102 registers where two CTAs share an SM (tc_ctas_per_sm): with more
+// only one fits, and the small layers take half as long again.
 template <int BN, int BKC, int STAGES, int G, int MT>
-__global__ void __launch_bounds__(TC_THREADS, 1)
+__global__ void __launch_bounds__(TC_THREADS, tc_ctas_per_sm(MT * BN))
     conv_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap,
                    const ConvArgs a, int ntiles, int ntn, int *err) {
     using S = TcSmem<BN, BKC, STAGES, G, MT>;
@@ -237,14 +255,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         }
                     }
                 }
-                if (a.out) {
+                if (a.out || a.act) {
                     uint4 o[2];
                     __nv_bfloat162 *h = reinterpret_cast<__nv_bfloat162 *>(o);
 #pragma unroll
                     for (int e = 0; e < 8; ++e) h[e] = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
-                    uint4 *dp = reinterpret_cast<uint4 *>(a.out + m * a.N + nb);
-                    dp[0] = o[0];
-                    dp[1] = o[1];
+                    if (a.zgrad) {
+                        uint4 zw[2];
+                        const uint4 *zp = reinterpret_cast<const uint4 *>(a.zgrad + m * a.N + nb);
+                        zw[0] = zp[0];
+                        zw[1] = zp[1];
+                        const __nv_bfloat162 *zh = reinterpret_cast<const __nv_bfloat162 *>(zw);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const float2 d = __bfloat1622float2(h[e]), z = __bfloat1622float2(zh[e]);
+                            h[e] = __floats2bfloat162_rn(silu_grad(d.x, z.x), silu_grad(d.y, z.y));
+                        }
+                    }
+                    if (a.out) {
+                        uint4 *dp = reinterpret_cast<uint4 *>(a.out + m * a.N + nb);
+                        dp[0] = o[0];
+                        dp[1] = o[1];
+                    }
                     if (a.act) {
 #pragma unroll
                         for (int e = 0; e < 8; ++e)
@@ -290,22 +322,6 @@ bool tile_for(int R, int P, TcTile *t) {
     t->Hy = R < P ? (R < P / R ? R : P / R) : 1;
     t->Bn = P / (t->Wx * t->Hy);
     return t->Wx * t->Hy * t->Bn == P && t->Wx <= 256 && t->Hy <= 256 && t->Bn <= 256;
-}
-
-// CTAs per SM and ring depth.  One thread issues a CTA's copies and one its
-// MMAs, and each ring slot costs them a few hundred cycles of issue and
-// barrier latency, so two CTAs per SM (two independent pipelines) run the
-// small layers about twice as fast as one CTA with a deeper ring, and a
-// slot carries as much work as its shared memory allows: two 32-channel K
-// steps (G = 2), or MT = 4 blocks of 128 pixels that share one weight box
-// (the 32-output-channel layers).  A ring takes about 104 KB of shared
-// memory per CTA (at most 16 slots); a CTA whose two accumulators fill
-// the 512 TMEM columns (BN = 256) runs alone on its SM with a 200 KB ring.
-constexpr int tc_ctas_per_sm(int acc_cols) { return 2 * acc_cols <= 256 ? 2 : 1; }
-constexpr int tc_stages(int stage, int acc_cols) {
-    return (tc_ctas_per_sm(acc_cols) == 2 ? 104 : 200) * 1024 / stage < 16
-               ? (tc_ctas_per_sm(acc_cols) == 2 ? 104 : 200) * 1024 / stage
-               : 16;
 }
 
 template <int BN, int BKC, int MT>
