@@ -47,8 +47,18 @@ constexpr int FAST_SLOTS = 4;
 constexpr int FAST_SLOTS_RHO0 = 3;
 constexpr int RHO0_NT = 128;
 
-template <bool RHO0>
+// Force field rows: every thread keeps its own column of Fx, Fy for rows
+// p-5 .. p+2 in shared memory, copied there two rows ahead (cp.async), because
+// the step needs each row's force three times (rows p, p-2, p-5) and a load of
+// it when it is needed puts an L2 round trip on the row's critical path: with
+// those loads and an integer modulo per use the forced march took 123 us a step
+// on 2048 x 1536 nodes in BF16, now 73.  The room comes from the TMA ring, so
+// that as many blocks fit an SM as without a force.
+constexpr int FORCE_ROWS = 8;
+
+template <bool FORCED, int ST, bool RHO0>
 __host__ __device__ constexpr int fast_slots() {
+    if (FORCED) return ST == STORAGE_FP32 ? 2 : 3;
     return RHO0 ? FAST_SLOTS_RHO0 : FAST_SLOTS;
 }
 
@@ -80,25 +90,26 @@ __device__ __forceinline__ W3 weights(float k, float step, const StepArgs &a) {
     return w;
 }
 
-// Force increment factor (step/5) (Fx, Fy) at a node, F_{j,alpha} = w_j F_alpha:
-// the h step's F, and the dt step's F + dt/2 dF/dt (Eq. 2.3.24).
-__device__ __forceinline__ F2 force_at(const StepArgs &a, int row, int X, F2 factor) {
-    if (a.force_mode == 0) return splat(0.0f);
-    if (a.force_mode == 1) return factor * mk2(a.Fx, a.Fy);
-    const long long fi = (long long)row * a.pitch + GHOST + X;
-    return factor * mk2(a.Fxp[fi], a.Fyp[fi]);
+// Four bytes from global to shared memory, asynchronously.
+__device__ __forceinline__ void cp_async4(void *dst, const float *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
-__device__ __forceinline__ F2 force_at_d(const StepArgs &a, int row, int X, F2 factor) {
-    if (a.force_mode_d == 0) return splat(0.0f);
-    if (a.force_mode_d == 1) return factor * mk2(a.Fxd, a.Fyd);
-    const long long fi = (long long)row * a.pitch + GHOST + X;
-    return factor * mk2(a.Fxdp[fi], a.Fydp[fi]);
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Row of the domain `back` rows before row p (0 <= p < ny, periodic).
+__device__ __forceinline__ int row_before(int p, int back, int ny) {
+    const int r = p - back;
+    return r < 0 ? r + ny : r;
 }
 
 template <int NT, int MK, bool FORCED, int ST, bool RHO0>
 __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
     fast_kernel(const __grid_constant__ CUtensorMap tmap, const StepArgs a) {
-    constexpr int SLOTS = fast_slots<RHO0>();
+    constexpr int SLOTS = fast_slots<FORCED, ST, RHO0>();
     // one TMA row: 10 FP32 planes (15 with alpha = 0), or u, v, P and 4
     // planes of 16-bit pairs
     constexpr int TROW = (RHO0 ? RHO0_PLANES : ST == STORAGE_FP32 ? NPLANES : DEV_PLANES) * NT * 4;
@@ -115,7 +126,12 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
     unsigned char *xB00 = ringP0 + RING * P0ROW;
     unsigned char *xF00 = xB00 + 2 * X0ROW;
     uint64_t *mbar = reinterpret_cast<uint64_t *>(xF00 + 2 * X0ROW);
-    __shared__ int s_abort;
+    unsigned char *ringF = reinterpret_cast<unsigned char *>(mbar + SLOTS);  // force field rows (FORCED)
+    // one flag per row parity: it is read after the barrier of its row, and a
+    // thread can set it again only two barriers later (a plain barrier and a
+    // load; with a voting barrier and the row index taken modulo ny by the
+    // copying thread the 4096^2 step took 279 us, now 267)
+    __shared__ volatile int s_abort[2];
 
     const int t = threadIdx.x;
     const int x0 = blockIdx.x * a.W;
@@ -128,18 +144,61 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
     constexpr bool forced = FORCED;
 
     if (t == 0) {
-        s_abort = 0;
+        s_abort[0] = s_abort[1] = 0;
         for (int i = 0; i < SLOTS; ++i) mbar_init(&mbar[i], 1);
         fence_mbar_init();
     }
     __syncthreads();
-    auto load_row = [&](int it, int slot) {
+    int rp = wrap(rowBase, a.ny);  // row p of the domain
+    int lrow = rp;                 // the next row to load
+    auto load_row = [&](int slot) {
         mbar_expect_tx(&mbar[slot], TROW);
-        tma_load_row(&tmap, &mbar[slot], tma + slot * TROW, x0, wrap(rowBase + it, a.ny));
+        tma_load_row(&tmap, &mbar[slot], tma + slot * TROW, x0, lrow);
+        lrow = lrow + 1 == a.ny ? 0 : lrow + 1;
     };
     int issued = min(SLOTS, nIt);
     if (t == 0)
-        for (int i = 0; i < issued; ++i) load_row(i, i);
+        for (int i = 0; i < issued; ++i) load_row(i);
+
+    // body force: F of this column for rows rp + 0, 1 (field), then two rows
+    // ahead of every row; the dt step reads the same rows unless a force rate
+    // gave it planes of its own
+    const bool ffield = FORCED && a.force_mode == 2;
+    const bool fd_same = ffield && a.force_mode_d == 2 && a.Fxdp == a.Fxp && a.Fydp == a.Fyp;
+    int frow = rp;  // the next force row to copy
+    auto force_slot = [&](int it) { return ringF + ((it & (FORCE_ROWS - 1)) * 2 * NT + t) * 4; };
+    auto copy_force = [&](int it) {
+        if (ffield && it < nIt) {
+            const long long e = (long long)frow * a.pitch + GHOST + X;
+            if (index_ok(a, e, a.plane)) {
+                cp_async4(force_slot(it), a.Fxp + e);
+                cp_async4(force_slot(it) + NT * 4, a.Fyp + e);
+            }
+            frow = frow + 1 == a.ny ? 0 : frow + 1;
+        }
+        cp_async_commit();
+    };
+    auto force_ring = [&](int it) {
+        const unsigned char *q = force_slot(it);
+        return mk2(lds1(q, 0), lds1(q, NT * 4));
+    };
+    // factor (Fx, Fy) of iteration row `it` in the h step (F_{j,alpha} = w_j
+    // F_alpha), and of output row r, iteration row `it`, in the dt step
+    // (F + dt/2 dF/dt, Eq. 2.3.24)
+    auto force_h = [&](int it, F2 factor) {
+        if (a.force_mode == 0) return splat(0.0f);
+        return factor * (ffield ? force_ring(it) : mk2(a.Fx, a.Fy));
+    };
+    auto force_dt = [&](int it, int r, F2 factor) {
+        if (a.force_mode_d == 0) return splat(0.0f);
+        if (fd_same) return factor * force_ring(it);
+        if (a.force_mode_d == 1) return factor * mk2(a.Fxd, a.Fyd);
+        return factor * field_pair(a, a.Fxdp, a.Fydp, (long long)r * a.pitch + GHOST + X);
+    };
+    if (FORCED) {
+        copy_force(0);
+        copy_force(1);
+    }
 
     W3 wxh, wxd;
     if (MK == METRIC_UNIFORM) {
@@ -183,7 +242,10 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
         constexpr int k = decltype(kc)::value;
         constexpr int s1 = (k + 4) % 5, s2 = (k + 3) % 5, s3 = (k + 2) % 5, s4 = (k + 1) % 5;
         {
-            const int p = rowBase + it;
+            if (FORCED) {
+                copy_force(it + 2);
+                cp_async_wait<2>();  // the copies of row p have landed
+            }
             // exchange buffers of this iteration (fbar^+) and of the previous one (f)
             unsigned char *xB = xB0 + (it & 1) * XROW;
             const unsigned char *xFp = xF0 + ((it & 1) ^ 1) * XROW;
@@ -194,13 +256,13 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
             // ---------------------------------------------- S0: output row r = p - 5
             if (it >= 9 && outc) {
                 // slot k of every window and of the ring holds row r
-                const int r = p - 5;
+                const int r = rowBase + it - 5;
                 const unsigned char *Pr = ringP + ps * PROW;
                 F2 out[5];
 #pragma unroll
                 for (int j = 0; j < 5; ++j) out[j] = lds2(Pr, (j * NT + t) * 8);
                 if (forced) {
-                    const F2 fF = force_at_d(a, r, X, pair_of(a.pdw));
+                    const F2 fF = force_dt(it - 5, r, pair_of(a.pdw));
 #pragma unroll
                     for (int j = 0; j < 5; ++j) out[j] = out[j] + fF;
                 }
@@ -242,14 +304,14 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
             float own01 = 0.0f, own03 = 0.0f;
             {
                 const bool ok = mbar_wait_bounded(&mbar[tslot], (uint32_t)((it / SLOTS) & 1));
-                if (!ok) atomicExch(&s_abort, 1);
+                if (!ok) s_abort[it & 1] = 1;
                 const float *src = reinterpret_cast<const float *>(tma + tslot * TROW);
                 F2 g[5], n[5], o[5];
                 if (ST == STORAGE_FP32) {
 #pragma unroll
                     for (int j = 0; j < 5; ++j) g[j] = mk2(src[j * NT + t], src[(5 + j) * NT + t]);
                     const Mom2 m = (forced && a.r_mode)
-                                       ? moments2r(g, c, a.rk_hat * source_at(a, wrap(p, a.ny), X))
+                                       ? moments2r(g, c, a.rk_hat * source_at(a, rp, X))
                                        : moments2(g, c);
                     noneq2(g, m, inv2c, n);
                     if (RHO0) {
@@ -298,10 +360,11 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
             // One barrier per row: the exchange rows are double-buffered, so
             // the buffers written before this barrier are read only after it,
             // and those read after it are rewritten only after the next one.
-            if (__syncthreads_or(s_abort)) return false;
+            __syncthreads();
+            if (s_abort[it & 1]) return false;
             if (t == 0 && issued < nIt) {
                 fence_proxy_async();
-                load_row(issued, tslot);
+                load_row(tslot);
                 ++issued;
             }
             tslot = (tslot == SLOTS - 1) ? 0 : tslot + 1;
@@ -327,7 +390,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
                 // pass 1, x part of row p: fbar = fbar^+ - h c.grad fbar^+ + h w F
                 F2 b1 = own1, b3 = own3;
                 if (forced) {
-                    const F2 hF = force_at(a, wrap(p, a.ny), X, pair_of(a.phw));
+                    const F2 hF = force_h(it, pair_of(a.phw));
                     D013[k][0] = D013[k][0] + hF;
                     b1 = b1 + hF;
                     b3 = b3 + hF;
@@ -340,7 +403,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
                     // the same on alpha = 0, with h w_j R
                     float b01 = own01, b03 = own03;
                     if (forced && a.r_mode) {
-                        const float sR = hw0 * source_at(a, wrap(p, a.ny), X);
+                        const float sR = hw0 * source_at(a, rp, X);
                         D0[k][0] += sR;
                         b01 += sR;
                         b03 += sR;
@@ -352,10 +415,10 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
                 }
                 if (it >= 4) {
                     // row q = p - 2 (slot s2); fbar^+ rows q-2..q+2 -> slots s4, s3, s2, s1, k
-                    const int qw = wrap(p - 2, a.ny);
+                    const int qw = row_before(rp, 2, a.ny);
                     F2 by2 = BY[s2][0], by4 = BY[s2][1];
                     if (forced) {
-                        const F2 hFq = force_at(a, qw, X, pair_of(a.phw));
+                        const F2 hFq = force_h(it - 2, pair_of(a.phw));
                         by2 = by2 + hFq;
                         by4 = by4 + hFq;
                     }
@@ -405,6 +468,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
                 }
             }
         }
+        rp = rp + 1 == a.ny ? 0 : rp + 1;
         return true;
     };
     // The march, unrolled by five so that every window slot is a
@@ -423,8 +487,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
         if (it0 + 4 >= nIt) break;
         if (!row(it0 + 4, integral_constant<int, 4>{}, 4)) { aborted = true; break; }
     }
-    (void)aborted;
-    if (s_abort) {
+    if (aborted) {
         if (t == 0) {
             for (int it = issued - SLOTS; it < issued; ++it) {
                 if (it < 0) continue;
@@ -435,18 +498,18 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
     }
 }
 
-template <int NT, int ST, bool RHO0>
+template <int NT, bool FORCED, int ST, bool RHO0>
 constexpr int fast_smem() {
-    return fast_slots<RHO0>() * (RHO0 ? RHO0_PLANES : ST == STORAGE_FP32 ? NPLANES : DEV_PLANES) * NT * 4 +
+    return fast_slots<FORCED, ST, RHO0>() * (RHO0 ? RHO0_PLANES : ST == STORAGE_FP32 ? NPLANES : DEV_PLANES) * NT * 4 +
            RING * 5 * NT * 8 + 4 * (2 * NT * 8) + (RHO0 ? RING * 5 * NT * 4 + 4 * (2 * NT * 4) : 0) +
-           fast_slots<RHO0>() * 8;
+           fast_slots<FORCED, ST, RHO0>() * 8 + (FORCED ? FORCE_ROWS * 2 * NT * 4 : 0);
 }
 
 template <int NT, int MK, bool FORCED, int ST, bool RHO0>
 cudaError_t fast_launch_t(const CUtensorMap *tmap, const StepArgs &args,
                           const StepPlan &plan, cudaStream_t stream) {
     auto k = fast_kernel<NT, MK, FORCED, ST, RHO0>;
-    constexpr int smem = fast_smem<NT, ST, RHO0>();
+    constexpr int smem = fast_smem<NT, FORCED, ST, RHO0>();
     static std::atomic<unsigned long long> configured{0};  // devices set up
     if (needs_device_setup(configured)) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -459,18 +522,19 @@ cudaError_t fast_launch_t(const CUtensorMap *tmap, const StepArgs &args,
 
 template <int NT, int MK, int ST, bool RHO0>
 cudaError_t fast_occupancy_t(int *occ, int *smem) {
-    // both force variants have the same shared memory; take the smaller occupancy
+    // the variant with a force trades TMA slots for force rows; report the
+    // larger shared memory and the smaller occupancy of the two
     int o1 = 0, o2 = 0;
-    *smem = fast_smem<NT, ST, RHO0>();
+    constexpr int s1 = fast_smem<NT, false, ST, RHO0>(), s2 = fast_smem<NT, true, ST, RHO0>();
+    *smem = s1 > s2 ? s1 : s2;
     cudaError_t e = cudaFuncSetAttribute(fast_kernel<NT, MK, false, ST, RHO0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, *smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, s1);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fast_kernel<NT, MK, true, ST, RHO0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 *smem);
+        e = cudaFuncSetAttribute(fast_kernel<NT, MK, true, ST, RHO0>, cudaFuncAttributeMaxDynamicSharedMemorySize, s2);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, fast_kernel<NT, MK, false, ST, RHO0>, NT, *smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, fast_kernel<NT, MK, false, ST, RHO0>, NT, s1);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, fast_kernel<NT, MK, true, ST, RHO0>, NT, *smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, fast_kernel<NT, MK, true, ST, RHO0>, NT, s2);
     *occ = o1 < o2 ? o1 : o2;
     return e;
 }
