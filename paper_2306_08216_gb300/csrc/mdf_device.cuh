@@ -127,6 +127,16 @@ __device__ __forceinline__ void tma_load_row(const CUtensorMap *map, uint64_t *b
         : "memory");
 }
 
+// Four bytes from global to shared memory, asynchronously.
+__device__ __forceinline__ void cp_async4(void *dst, const float *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // ------------------------------------------------------------ local maps
 
 // Node in pair form: g[j] = (g_{j,u}, g_{j,v}), j = 0..4.
@@ -360,24 +370,74 @@ __device__ __forceinline__ float stream1(float base, float pf, float p0, float p
     return fmaf(w1, pf - pb1, fmaf(w0, d0, fmaf(w2, dfar, base)));
 }
 
-// Rotate a register window by one row for a rolled march (the register-
-// window marches that keep their loop rolled).  Its window slots follow the slot formula of the unrolled march with the slot of the
-// newest row p fixed at 0: row p - a sits in slot (5 - a) mod 5 (row p - 1 in
-// slot 4, ..., row p - 4 in slot 1, and slot 0 before the write of row p
-// still holds row p - 5).  Advancing p moves every row to the slot below it
-// (modulo 5): new[i] = old[(i + 1) mod 5].
-template <typename T, int N>
-__device__ __forceinline__ void rot5(T (&w)[5][N]) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        const T w0 = w[0][i];
-        w[0][i] = w[1][i];
-        w[1][i] = w[2][i];
-        w[2][i] = w[3][i];
-        w[3][i] = w[4][i];
-        w[4][i] = w0;
-    }
+// stream2 / stream1 in two parts: the sum without its foremost point, then
+// that point.
+template <bool WALLS>
+__device__ __forceinline__ F2 stream_tail(F2 base, F2 p0, F2 pb1, F2 pb2, bool wall_adj, F2 w0, F2 w2) {
+    const F2 d0 = p0 - pb1;
+    F2 dfar = pb2 - pb1;
+    if (WALLS) dfar = sel2(wall_adj, splat(0.0f) - d0, dfar);
+    return fma2(w0, d0, fma2(w2, dfar, base));
 }
+template <bool WALLS>
+__device__ __forceinline__ float stream_tail(float base, float p0, float pb1, float pb2, bool wall_adj, float w0,
+                                             float w2) {
+    const float d0 = p0 - pb1;
+    float dfar = pb2 - pb1;
+    if (WALLS && wall_adj) dfar = -d0;
+    return fmaf(w0, d0, fmaf(w2, dfar, base));
+}
+__device__ __forceinline__ F2 stream_head(F2 pf, F2 pb1, F2 tail, F2 w1) { return fma2(w1, pf - pb1, tail); }
+__device__ __forceinline__ float stream_head(float pf, float pb1, float tail, float w1) {
+    return fmaf(w1, pf - pb1, tail);
+}
+template <bool WALLS>
+__device__ __forceinline__ F2 stream(F2 base, F2 pf, F2 p0, F2 pb1, F2 pb2, bool adj, F2 w1, F2 w0, F2 w2) {
+    return stream2<WALLS>(base, pf, p0, pb1, pb2, adj, w1, w0, w2);
+}
+template <bool WALLS>
+__device__ __forceinline__ float stream(float base, float pf, float p0, float pb1, float pb2, bool adj, float w1,
+                                        float w0, float w2) {
+    return stream1<WALLS>(base, pf, p0, pb1, pb2, adj, w1, w0, w2);
+}
+
+// What a march's y stencils (populations 2 and 4) keep of the rows before the
+// newest one, in registers: with newest row p and completed row q = p - 2,
+//   population 2 (moving +y) reads rows q-2 .. q+1, so its sum is begun when row
+//   q is the newest (every term but the foremost) and completed one row later:
+//   rows p-1 and p-2, the sum begun for row p-1, the result of row p-2;
+//   population 4 (moving -y) reads rows q-1 .. q+2: rows p-1, p-2, p-3.
+// Seven values and a handful of moves per row, where a window of five rows per
+// population holds ten and has to be unrolled five times (a code of five
+// bodies) or rotated (twenty moves).  The operations and their order are those
+// of stream2 / stream1.
+template <typename T>
+struct YCarry {
+    T a2, b2, sum2, done2;  // population 2: rows p-1, p-2, begun sum, completed row
+    T a4, b4, c4;           // population 4: rows p-1, p-2, p-3
+    __device__ __forceinline__ void clear(T zero) { a2 = b2 = sum2 = done2 = a4 = b4 = c4 = zero; }
+    // result of population 2 in row q (completed when row p-1 arrived)
+    __device__ __forceinline__ T two() const { return done2; }
+    // result of population 4 in row q: base (its value there plus the force),
+    // n4 the newest row; adj: row q lies next to a wall it moves towards
+    template <bool WALLS, typename W>
+    __device__ __forceinline__ T four(T base, T n4, bool adj, const W &w) const {
+        return stream<WALLS>(base, c4, b4, a4, n4, adj, w.w1, w.w0, w.w2);
+    }
+    // take up row p: n2, n4 its values, base the value population 2 is
+    // streamed onto there, wp / wm the weights of rows p / p-1; adj: row p lies
+    // next to a wall population 2 moves away from
+    template <bool WALLS, typename W>
+    __device__ __forceinline__ void push(T n2, T n4, T base, bool adj, const W &wp, const W &wm) {
+        done2 = stream_head(n2, b2, sum2, wm.w1);
+        sum2 = stream_tail<WALLS>(base, n2, a2, b2, adj, wp.w0, wp.w2);
+        b2 = a2;
+        a2 = n2;
+        c4 = b4;
+        b4 = a4;
+        a4 = n4;
+    }
+};
 
 __device__ __forceinline__ int wrap(int i, int n) {
     i %= n;

@@ -90,16 +90,6 @@ __device__ __forceinline__ W3 weights(float k, float step, const StepArgs &a) {
     return w;
 }
 
-// Four bytes from global to shared memory, asynchronously.
-__device__ __forceinline__ void cp_async4(void *dst, const float *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // Row of the domain `back` rows before row p (0 <= p < ny, periodic).
 __device__ __forceinline__ int row_before(int p, int back, int ny) {
     const int r = p - back;
