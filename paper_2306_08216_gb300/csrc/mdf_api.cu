@@ -1080,6 +1080,9 @@ mdf_status mdf_set_launch(mdf_ctx *c, int threads, int rows_per_block) {
         const bool tile = c->cand[i].kind == PLAN_TILE;
         if (threads == 0 ? tile : (!tile && c->cand[i].NT == threads)) { found = i; break; }
     }
+    // tiles of rows_per_block rows where the problem has a plan of them
+    for (int i = 0; threads == 0 && i < c->ncand; ++i)
+        if (c->cand[i].kind == PLAN_TILE && c->cand[i].H == rows_per_block) found = i;
     if (found < 0) return fail(c, MDF_E_INVALID, "no launch plan with %d threads for this problem", threads);
     if (threads != 0 && rows_per_block < 1) return fail(c, MDF_E_INVALID, "rows_per_block must be >= 1");
     StepPlan p = c->cand[found];

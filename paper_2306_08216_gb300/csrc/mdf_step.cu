@@ -101,15 +101,23 @@ int step_candidates(int metric, int power_law, int walls, int storage, int rho0,
             return n;
         }
         if (occ >= 1) {
-            StepPlan &p = out[n++];
-            p.kind = PLAN_TILE;
-            p.NT = tx * ty;
-            p.W = tx;
-            p.H = ty;
-            p.gx = (nx + tx - 1) / tx;
-            p.gy = (ny + ty - 1) / ty;
-            p.smem = smem;
-            p.occ = occ;
+            const auto tile_plan = [&](int tw, int th) {
+                StepPlan &p = out[n++];
+                p.kind = PLAN_TILE;
+                p.NT = tx * ty;
+                p.W = tw;
+                p.H = th;
+                p.gx = (nx + tw - 1) / tw;
+                p.gy = (ny + th - 1) / th;
+                p.smem = smem;
+                p.occ = occ;
+            };
+            tile_plan(tx, ty);
+            // 8 x 8 tiles while a grid of them still fits the SMs at three
+            // blocks each: from about there on their larger halo costs more than
+            // the shorter phases give
+            const long long small = (long long)((nx + 7) / 8) * ((ny + 7) / 8);
+            if (storage == STORAGE_FP32 && !rho0 && n < max && small <= 3ll * (num_sms > 0 ? num_sms : 1)) tile_plan(8, 8);
         }
     }
     return n;

@@ -53,9 +53,20 @@ __device__ __forceinline__ int axis_index(int i, int n, bool wall) {
     return wrap(i, n);
 }
 
+// Threads of a block: one per output node on the 16 x 16 tile; on the 8 x 8
+// tile the same 256, one per node of the 16 x 16 region of phase A, so that each
+// phase is a single pass.  The small tile recomputes more (4 and 2.25 times the
+// output in phases A and B, against 2.25 and 1.56), which costs nothing on a
+// grid that leaves most SMs without a block, where the length of a block's three
+// phases is the time of the step (64^2 periodic nodes, 16 -> 64
+// blocks: 3.72 -> 2.56 us a step).
+constexpr int kTileThreads = 256;
+constexpr int kSmallTile = 8;
+
 template <int TX, int TY>
 struct Tile {
-    static constexpr int NT = TX * TY;
+    static constexpr int NT = kTileThreads;
+    static constexpr int N0 = TX * TY;  // output nodes
     static constexpr int X8 = TX + 8, Y8 = TY + 8, N8 = X8 * Y8;  // fbar^+ region: tile + 4
     static constexpr int X4 = TX + 4, Y4 = TY + 4, N4 = X4 * Y4;  // f region: tile + 2
     static constexpr int B_BYTES = 5 * N8 * 8;
@@ -211,12 +222,12 @@ __device__ __forceinline__ void tile_step(const StepArgs &a, int bx, int by, uns
     // share one memory latency.
     constexpr int PASSES = (T::N8 + T::NT - 1) / T::NT;
     auto region_node = [&](int i, int &lx, int &ly) {
-        if (i < T::NT) {
+        if (i < T::N0) {
             lx = 4 + i % TX;
             ly = 4 + i / TX;
             return;
         }
-        int h = i - T::NT;
+        int h = i - T::N0;
         if (h < 4 * T::X8) {
             ly = h / T::X8;
             lx = h % T::X8;
@@ -432,6 +443,7 @@ __device__ __forceinline__ void tile_step(const StepArgs &a, int bx, int by, uns
     // ------------------------------------------------ C: fhat(t+dt) of the own node
     const int li = t % TX, lj = t / TX;
     const int X = x0 + li, Y = y0 + lj;
+    if (T::N0 < T::NT && t >= T::N0) return;
     if (X >= a.nx || Y >= a.ny) return;
     if (WALLS && ((xwall && (X == 0 || X == a.nx - 1)) || (ywall && (Y == 0 || Y == a.ny - 1)))) return;
     tile_output<TX, TY, MK, WALLS, ST, RHO0>(a, X, Y, li, lj, Fs, Fs0, hp, hp0);
@@ -518,7 +530,7 @@ __device__ __forceinline__ void tile_output(const StepArgs &a, int X, int Y, int
 }
 
 template <int TX, int TY, int MK, bool PL, bool WALLS, int ST, bool RHO0>
-__global__ void __launch_bounds__(TX *TY, kTileMinBlocks) tile_kernel(const StepArgs a) {
+__global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) tile_kernel(const StepArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     // launched with programmatic stream serialization: the block touches
     // global memory only after the previous step has completed.  The next
@@ -532,7 +544,7 @@ __global__ void __launch_bounds__(TX *TY, kTileMinBlocks) tile_kernel(const Step
 // Many problems in one persistent launch: block b steps work items
 // b, b + gridDim.x, ... (problem, tile x, tile y), largest problems first.
 template <int TX, int TY, int MK, bool PL, bool WALLS, int ST>
-__global__ void __launch_bounds__(TX *TY, kTileMinBlocks) tile_batch_kernel(const BatchItem *__restrict__ items, int nitems,
+__global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) tile_batch_kernel(const BatchItem *__restrict__ items, int nitems,
                                                                const StepArgs *__restrict__ args) {
     extern __shared__ __align__(128) unsigned char smem[];
     for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
@@ -543,9 +555,9 @@ __global__ void __launch_bounds__(TX *TY, kTileMinBlocks) tile_batch_kernel(cons
 
 constexpr int kTX = TILE_X, kTY = TILE_Y;
 
-template <int MK, bool PL, bool WALLS, bool RHO0 = false>
+template <int MK, bool PL, bool WALLS, bool RHO0 = false, int TS = kTX>
 constexpr int tile_smem() {
-    using T = Tile<kTX, kTY>;
+    using T = Tile<TS, TS>;
     return T::B_BYTES + T::F_BYTES + (PL ? T::K_BYTES : 0) + (RHO0 ? T::B0_BYTES + T::F0_BYTES : 0);
 }
 
@@ -555,13 +567,14 @@ cudaError_t tile_occupancy_t(int *occ, int *smem) {
     *smem = tile_smem<MK, PL, WALLS, RHO0>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, kTX * kTY, *smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, kTileThreads, *smem);
 }
 
-template <int MK, bool PL, bool WALLS, int ST, bool RHO0 = false>
-cudaError_t tile_launch_t(const StepArgs &args, const StepPlan &plan, cudaStream_t stream) {
-    auto k = tile_kernel<kTX, kTY, MK, PL, WALLS, ST, RHO0>;
-    constexpr int smem = tile_smem<MK, PL, WALLS, RHO0>();
+// One step with tiles of TS x TS nodes.
+template <int MK, bool PL, bool WALLS, int ST, bool RHO0, int TS>
+cudaError_t tile_launch_ts(const StepArgs &args, const StepPlan &plan, cudaStream_t stream) {
+    auto k = tile_kernel<TS, TS, MK, PL, WALLS, ST, RHO0>;
+    constexpr int smem = tile_smem<MK, PL, WALLS, RHO0, TS>();
     static std::atomic<unsigned long long> configured{0};  // devices set up
     if (needs_device_setup(configured)) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -572,7 +585,7 @@ cudaError_t tile_launch_t(const StepArgs &args, const StepPlan &plan, cudaStream
     // scheduled while this one drains (tile_kernel waits for it in hardware)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(plan.gx, plan.gy);
-    cfg.blockDim = dim3(kTX * kTY);
+    cfg.blockDim = dim3(kTileThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -585,13 +598,23 @@ cudaError_t tile_launch_t(const StepArgs &args, const StepPlan &plan, cudaStream
     return cudaGetLastError();
 }
 
+// The small tile serves FP32 storage without the alpha = 0 lane.
+template <int MK, bool PL, bool WALLS, int ST, bool RHO0 = false>
+cudaError_t tile_launch_t(const StepArgs &args, const StepPlan &plan, cudaStream_t stream) {
+    if constexpr (ST == STORAGE_FP32 && !RHO0) {
+        if (plan.W == kSmallTile) return tile_launch_ts<MK, PL, WALLS, ST, RHO0, kSmallTile>(args, plan, stream);
+    }
+    if (plan.W != kTX) return cudaErrorInvalidConfiguration;
+    return tile_launch_ts<MK, PL, WALLS, ST, RHO0, kTX>(args, plan, stream);
+}
+
 template <int MK, bool PL, bool WALLS, int ST>
 cudaError_t tile_batch_occupancy_t(int *occ, int *smem) {
     auto k = tile_batch_kernel<kTX, kTY, MK, PL, WALLS, ST>;
     *smem = tile_smem<MK, PL, WALLS>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, kTX * kTY, *smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, kTileThreads, *smem);
 }
 
 template <int MK, bool PL, bool WALLS, int ST>
@@ -604,7 +627,7 @@ cudaError_t tile_batch_launch_t(const BatchItem *items, int nitems, const StepAr
         if (e != cudaSuccess) return e;
         mark_device_setup(configured);
     }
-    k<<<grid, kTX * kTY, tile_smem<MK, PL, WALLS>(), stream>>>(items, nitems, args);
+    k<<<grid, kTileThreads, tile_smem<MK, PL, WALLS>(), stream>>>(items, nitems, args);
     return cudaGetLastError();
 }
 
