@@ -337,7 +337,7 @@ double mdf_bytes_per_node(const mdf_ctx *ctx);
  * A batch holds `count` independent problems (each an ordinary context with
  * its own grid, fluid, walls and scheme parameters) and advances them
  * together: each time step is ONE launch whose blocks walk a table of work
- * items (problem, strip, band), largest problems first, reading each
+ * items (problem, strip, band), longest bands first, reading each
  * problem's arguments and TMA descriptor from device memory; repeated steps
  * are replayed from captured CUDA graphs.  All problems must share the grid
  * kind, the fluid model (Newtonian or power law) and the wall/periodic type

@@ -18,6 +18,7 @@
 
 #include <algorithm>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "mdf_ctx.cuh"
@@ -25,7 +26,6 @@
 using namespace mdf;
 
 namespace {
-constexpr int kBandRows = 128;    // longest band (rows per work item)
 constexpr int kGraphSteps = 16;   // launches per captured graph (even: parity returns)
 }  // namespace
 
@@ -37,7 +37,9 @@ struct mdf_batch {
     CUtensorMap *d_maps[2] = {nullptr, nullptr};   // per parity: maps of the input buffer
     BatchItem *d_items = nullptr;
     int nt = 0;                                    // block size of the march kernel (strips of nt - 8 columns)
+    int *d_queue = nullptr;                        // the marches' next item and finished blocks
     int nitems = 0, grid = 0, occ = 0, smem = 0;
+    bool bands_chosen = false;                     // H holds the band heights of the active set
     int tile = 0, occ_tile = 0, smem_tile = 0;     // tile mode: one work item per 16 x 16 tile
     int roll = 0;                                  // march mode: the rolled register-window march
     int pinned = 0;                                // mode set by mdf_batch_set_launch (no re-timing)
@@ -86,6 +88,7 @@ static void free_batch(mdf_batch *b) {
         if (b->d_maps[p]) cudaFree(b->d_maps[p]);
     }
     if (b->d_items) cudaFree(b->d_items);
+    if (b->d_queue) cudaFree(b->d_queue);
     if (b->h_res) cudaFreeHost(b->h_res);
     if (b->ev_in) cudaEventDestroy(b->ev_in);
     if (b->ev_out) cudaEventDestroy(b->ev_out);
@@ -136,7 +139,7 @@ static cudaError_t launch_one(mdf_batch *b, int parity, cudaStream_t st) {
     if (b->tile)
         return tile_batch_launch(b->d_items, b->nitems, b->d_args[parity], b->metric, b->power_law, b->walls,
                                  b->storage, b->grid, st);
-    return batch_launch(b->d_items, b->nitems, b->d_args[parity], b->d_maps[parity], b->metric, b->power_law,
+    return batch_launch(b->d_items, b->nitems, b->d_queue, b->d_args[parity], b->d_maps[parity], b->metric, b->power_law,
                         b->walls, b->grid, b->forced, b->roll, b->storage, st);
 }
 
@@ -167,56 +170,126 @@ static mdf_status build_graph(mdf_batch *b, int parity) {
     return MDF_OK;
 }
 
-// Work items of the active problems, largest problems first, with band
-// heights sized to the active work: a band of H rows costs H + 9 row
-// iterations (halo), so long bands are cheapest when there is enough work to
-// fill every resident block; a small batch instead gets bands short enough
-// that its items cover the grid (one item per block, at least 2 rows).
-static mdf_status build_items(mdf_batch *b) {
-    const int count = b->count;
-    const int W = b->nt - 8;
-    long long strip_rows = 0;
-    for (int i = 0; i < count; ++i)
-        if (b->active[i]) strip_rows += (long long)((b->ctx[i]->nx + W - 1) / W) * b->ctx[i]->ny;
-    const long long slots = (long long)std::max(1, b->occ) * b->num_sms;
-    const int band_target = (int)std::max(2ll, std::min((long long)kBandRows, (strip_rows + slots - 1) / slots));
-    for (int i = 0; i < count; ++i) {
-        const int ny = b->ctx[i]->ny;
-        const int bands = (ny + band_target - 1) / band_target;
-        int H = (ny + bands - 1) / bands;
-        if (H < 2) H = 2;
-        b->H[i] = H;
-    }
-    std::vector<int> order;
-    std::vector<BatchItem> items;
-    try {
-        for (int i = 0; i < count; ++i)
-            if (b->active[i]) order.push_back(i);
-        std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-            return (long long)b->ctx[x]->nx * b->ctx[x]->ny > (long long)b->ctx[y]->nx * b->ctx[y]->ny;
-        });
-        for (int i : order) {
-            mdf_ctx *c = b->ctx[i];
-            const int tw = b->tile ? TILE_X : W, th = b->tile ? TILE_Y : b->H[i];
-            const int gx = (c->nx + tw - 1) / tw;
-            const int gy = (c->ny + th - 1) / th;
-            for (int by = 0; by < gy; ++by)
-                for (int bx = 0; bx < gx; ++bx) items.push_back(BatchItem{i, bx, by, 0});
+// Rows of every band when a band has about `target` of them.
+static int band_rows(int ny, int target) {
+    const int bands = (ny + target - 1) / target;
+    const int H = (ny + bands - 1) / bands;
+    return H < 2 ? 2 : H;
+}
+
+// Row iterations of the march over a band of `rows` rows: its halo of eight and
+// about three more for the copies to arrive.
+static int band_work(int rows) { return rows + 11; }
+
+// Longest block when every block takes the next item as it finishes one (items:
+// number of row iterations and how many such items, in order).
+static long long longest_block(const std::vector<std::pair<int, long long>> &items, int blocks) {
+    std::vector<long long> heap(blocks, 0);
+    const auto later = [](long long x, long long y) { return x > y; };
+    long long longest = 0;
+    for (const auto &it : items)
+        for (long long k = 0; k < it.second; ++k) {
+            std::pop_heap(heap.begin(), heap.end(), later);
+            heap.back() += it.first;
+            longest = std::max(longest, heap.back());
+            std::push_heap(heap.begin(), heap.end(), later);
         }
+    return longest;
+}
+
+// The active problems, largest first.
+static std::vector<int> problem_order(const mdf_batch *b) {
+    std::vector<int> order;
+    for (int i = 0; i < b->count; ++i)
+        if (b->active[i]) order.push_back(i);
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+        return (long long)b->ctx[x]->nx * b->ctx[x]->ny > (long long)b->ctx[y]->nx * b->ctx[y]->ny;
+    });
+    return order;
+}
+
+// Band heights of the active problems.  Long bands spend the least on halo
+// rows; with few items per block a step waits for the blocks that got one more
+// (96 cavities of 65^2 to 513^2 in bands of 128 rows: 1056 items for 760
+// blocks).  The blocks left over run faster as their neighbours finish: a step's
+// time follows the mean work per block and, measured, a fifth of what the
+// longest block has above it; the target height with the least of that sum is
+// taken (bands of 128 rows -> chosen: 48 cavities 194 -> 171 us a step, 96 392 ->
+// 317; from 256 cavities on 128 rows are the best).
+static void choose_bands(mdf_batch *b) {
+    static const int targets[] = {128, 112, 96, 80, 64, 48, 40, 32, 24, 16, 12, 8, 6, 4, 3, 2};
+    const int blocks = std::max(1, b->occ) * b->num_sms, W = b->nt - 8;
+    const std::vector<int> order = problem_order(b);
+    std::vector<int> H(b->count, 2);
+    std::vector<std::pair<int, long long>> items;
+    double best = -1.0;
+    for (const int target : targets) {
+        long long n = 0, work = 0;
+        items.clear();
+        for (const int i : order) {
+            const long long strips = (b->ctx[i]->nx + W - 1) / W;
+            const int ny = b->ctx[i]->ny;
+            H[i] = band_rows(ny, target);
+            const int full = ny / H[i], rest = ny % H[i];
+            if (full) items.push_back(std::make_pair(band_work(H[i]), full * strips));
+            if (rest) items.push_back(std::make_pair(band_work(rest), strips));
+            n += (full + (rest ? 1 : 0)) * strips;
+            work += ((long long)full * band_work(H[i]) + (rest ? band_work(rest) : 0)) * strips;
+        }
+        // from five items per block on the longest bands are the best
+        if (best < 0) b->H = H;
+        if (n > 5ll * blocks || n == 0) break;
+        std::stable_sort(items.begin(), items.end(),
+                         [](const std::pair<int, long long> &x, const std::pair<int, long long> &y) {
+                             return x.first > y.first;
+                         });
+        const double cost = 0.8 * (double)work / blocks +
+                            0.2 * (double)longest_block(items, (int)std::min((long long)blocks, n));
+        if (best < 0 || cost < best) {
+            best = cost;
+            b->H = H;
+        }
+    }
+    b->bands_chosen = true;
+}
+
+// Work items of the active problems, longest first: marches by the rows of the
+// band (their blocks take the next item as they finish one), tiles by problem.
+static mdf_status build_items(mdf_batch *b) {
+    std::vector<std::pair<int, BatchItem>> items;
+    std::vector<BatchItem> table;
+    try {
+        if (!b->bands_chosen) choose_bands(b);
+        const int W = b->nt - 8;
+        for (const int i : problem_order(b)) {
+            const mdf_ctx *c = b->ctx[i];
+            const int tw = b->tile ? TILE_X : W, th = b->tile ? TILE_Y : b->H[i];
+            const int gx = (c->nx + tw - 1) / tw, gy = (c->ny + th - 1) / th;
+            for (int by = 0; by < gy; ++by) {
+                const int rows = std::min(th, c->ny - by * th);
+                for (int bx = 0; bx < gx; ++bx)
+                    items.push_back(std::make_pair(b->tile ? 0 : rows, BatchItem{i, bx, by, 0}));
+            }
+        }
+        std::stable_sort(items.begin(), items.end(),
+                         [](const std::pair<int, BatchItem> &x, const std::pair<int, BatchItem> &y) {
+                             return x.first > y.first;
+                         });
+        for (const auto &it : items) table.push_back(it.second);
     } catch (const std::bad_alloc &) {
         return bfail(b, MDF_E_NOMEM, "host allocation of the work items failed");
     }
-    b->nitems = (int)items.size();
+    b->nitems = (int)table.size();
     b->grid = std::min(b->nitems, std::max(1, b->tile ? b->occ_tile : b->occ) * b->num_sms);
     if (b->nitems > b->items_cap) {
         if (b->d_items) cudaFree(b->d_items);
         b->d_items = nullptr;
         b->items_cap = 0;
-        BCK(b, cudaMalloc(&b->d_items, items.size() * sizeof(BatchItem)));
+        BCK(b, cudaMalloc(&b->d_items, table.size() * sizeof(BatchItem)));
         b->items_cap = b->nitems;
     }
     if (b->nitems)
-        BCK(b, cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice));
+        BCK(b, cudaMemcpy(b->d_items, table.data(), table.size() * sizeof(BatchItem), cudaMemcpyHostToDevice));
     for (int p = 0; p < 2; ++p) {
         if (b->graph[p]) cudaGraphExecDestroy(b->graph[p]);
         b->graph[p] = nullptr;
@@ -355,6 +428,9 @@ mdf_status mdf_batch_create(int count, const mdf_grid *grids, const mdf_fluid *f
         for (int p = 0; p < 2; ++p) b->h_maps[p][i] = m[p];
     }
     BCKC(build_items(b));
+    BCKE(cudaMalloc(&b->d_queue, 2 * sizeof(int)));
+    BCKE(cudaMemset(b->d_queue, 0, 2 * sizeof(int)));
+    BCKE(cudaStreamSynchronize(nullptr));
     for (int p = 0; p < 2; ++p) {
         BCKE(cudaMalloc(&b->d_args[p], count * sizeof(StepArgs)));
         BCKE(cudaMalloc(&b->d_maps[p], count * sizeof(CUtensorMap)));
@@ -470,6 +546,7 @@ mdf_status mdf_batch_set_active(mdf_batch *b, int index, int active) {
                               cudaMemcpyHostToDevice));
     }
     b->active[index] = (char)active;
+    b->bands_chosen = false;
     mdf_status s = build_items(b);
     if (s != MDF_OK) return s;
     s = upload_args(b);

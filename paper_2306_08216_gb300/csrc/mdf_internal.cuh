@@ -158,7 +158,7 @@ struct BatchItem {
 // only, rolled form).  roll: the rolled form of the register-window march
 // (uniform and separable grids; ignored on curvilinear grids).
 cudaError_t batch_occupancy(int metric, int power_law, int walls, int storage, int *nt, int *occ, int *smem);
-cudaError_t batch_launch(const BatchItem *items, int nitems, const StepArgs *args, const CUtensorMap *maps, int metric,
+cudaError_t batch_launch(const BatchItem *items, int nitems, int *queue, const StepArgs *args, const CUtensorMap *maps, int metric,
                          int power_law, int walls, int grid, int forced, int roll, int storage, cudaStream_t stream);
 
 // Walls and/or power law on uniform/separable grids, FP32 storage, in the
@@ -168,12 +168,12 @@ cudaError_t walls_occupancy(int metric, int power_law, int nt, int *occ, int *sm
 cudaError_t walls_launch(const CUtensorMap *tmap, const StepArgs &args, int metric, const StepPlan &plan,
                          cudaStream_t stream);
 cudaError_t walls_batch_occupancy(int metric, int power_law, int storage, int *nt, int *occ, int *smem);
-cudaError_t walls_batch_launch(const BatchItem *items, int nitems, const StepArgs *args, const CUtensorMap *maps,
+cudaError_t walls_batch_launch(const BatchItem *items, int nitems, int *queue, const StepArgs *args, const CUtensorMap *maps,
                                int metric, int power_law, int grid, int forced, int roll, int storage,
                                cudaStream_t stream);
 // The 16-bit batched wall march (FP16/BF16 storage, rolled form only).
 cudaError_t walls_batch_occupancy16(int metric, int power_law, int storage, int *occ, int *smem);
-cudaError_t walls_batch_launch16(const BatchItem *items, int nitems, const StepArgs *args, const CUtensorMap *maps,
+cudaError_t walls_batch_launch16(const BatchItem *items, int nitems, int *queue, const StepArgs *args, const CUtensorMap *maps,
                                  int metric, int power_law, int grid, int forced, int roll, int storage,
                                  cudaStream_t stream);
 

@@ -672,20 +672,19 @@ __global__ void __launch_bounds__(NT) step_kernel(const __grid_constant__ CUtens
     march<NT, MK, PL, WALLS, RHO0>(&tmap, a, blockIdx.x, blockIdx.y, smem, &s_abort);
 }
 
-// Many problems in one persistent launch: block b takes work items
-// b, b + gridDim.x, ... of the table (problem, strip, band), which lists the
-// largest problems first.  Arguments and TMA descriptors live in global memory.
+// Many problems in one persistent launch: the blocks take the items of the table
+// (problem, strip, band; longest bands first) one after the other (each_item).
+// Arguments and TMA descriptors live in global memory.
 template <int NT, int MK, bool PL, bool WALLS, bool RHO0>
-__global__ void __launch_bounds__(NT) batch_kernel(const BatchItem *__restrict__ items, int nitems,
+__global__ void __launch_bounds__(NT) batch_kernel(const BatchItem *__restrict__ items, int nitems, int *queue,
                                                    const StepArgs *__restrict__ args,
                                                    const CUtensorMap *__restrict__ maps) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_abort;
-    for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
-        const BatchItem item = items[w];
+    each_item(items, nitems, queue, [&](const BatchItem &item) {
         march<NT, MK, PL, WALLS, RHO0>(&maps[item.problem], args[item.problem], item.bx, item.by, smem, &s_abort);
-        if (s_abort) break;
-    }
+        return s_abort == 0;
+    });
 }
 
 template <int NT, int MK, bool PL, bool WALLS, bool RHO0>
@@ -718,7 +717,7 @@ cudaError_t occupancy_t(int *occ, int *smem) {
 }
 
 template <int NT, int MK, bool PL, bool WALLS, bool RHO0>
-cudaError_t batch_launch_t(const BatchItem *items, int nitems, const StepArgs *args, const CUtensorMap *maps,
+cudaError_t batch_launch_t(const BatchItem *items, int nitems, int *queue, const StepArgs *args, const CUtensorMap *maps,
                            int grid, cudaStream_t stream) {
     auto k = batch_kernel<NT, MK, PL, WALLS, RHO0>;
     const int smem = smem_bytes<NT, MK, PL, WALLS, RHO0>();
@@ -728,7 +727,7 @@ cudaError_t batch_launch_t(const BatchItem *items, int nitems, const StepArgs *a
         if (e != cudaSuccess) return e;
         mark_device_setup(configured);
     }
-    k<<<grid, NT, smem, stream>>>(items, nitems, args, maps);
+    k<<<grid, NT, smem, stream>>>(items, nitems, queue, args, maps);
     return cudaGetLastError();
 }
 

@@ -129,11 +129,11 @@ cudaError_t batch_occupancy(int metric, int power_law, int walls, int storage, i
     MDF_CURVI_DISPATCH(batch_occupancy_t, occ, smem)
 }
 
-cudaError_t batch_launch(const BatchItem *items, int nitems, const StepArgs *args, const CUtensorMap *maps, int metric,
+cudaError_t batch_launch(const BatchItem *items, int nitems, int *queue, const StepArgs *args, const CUtensorMap *maps, int metric,
                          int power_law, int walls, int grid, int forced, int roll, int storage, cudaStream_t stream) {
     if (metric != METRIC_CURVILINEAR)
-        return walls_batch_launch(items, nitems, args, maps, metric, power_law, grid, forced, roll, storage, stream);
-    MDF_CURVI_DISPATCH(batch_launch_t, items, nitems, args, maps, grid, stream)
+        return walls_batch_launch(items, nitems, queue, args, maps, metric, power_law, grid, forced, roll, storage, stream);
+    MDF_CURVI_DISPATCH(batch_launch_t, items, nitems, queue, args, maps, grid, stream)
 }
 
 cudaError_t step_launch(const CUtensorMap *tmap, const StepArgs &args, int metric, const StepPlan &plan,

@@ -28,12 +28,12 @@ cudaError_t walls_batch_occupancy(int metric, int power_law, int storage, int *n
     MDF_WALLS_DISPATCH_ST(kWallsBatchNT, STORAGE_FP32, batch_occupancy_t, occ, smem)
 }
 
-cudaError_t walls_batch_launch(const BatchItem *items, int nitems, const StepArgs *args, const CUtensorMap *maps,
+cudaError_t walls_batch_launch(const BatchItem *items, int nitems, int *queue, const StepArgs *args, const CUtensorMap *maps,
                                int metric, int power_law, int grid, int forced, int roll, int storage,
                                cudaStream_t stream) {
     if (storage != STORAGE_FP32)
-        return walls_batch_launch16(items, nitems, args, maps, metric, power_law, grid, forced, roll, storage, stream);
-    MDF_WALLS_DISPATCH_ST(kWallsBatchNT, STORAGE_FP32, batch_launch_t, items, nitems, args, maps, grid, forced, roll,
+        return walls_batch_launch16(items, nitems, queue, args, maps, metric, power_law, grid, forced, roll, storage, stream);
+    MDF_WALLS_DISPATCH_ST(kWallsBatchNT, STORAGE_FP32, batch_launch_t, items, nitems, queue, args, maps, grid, forced, roll,
                           stream)
 }
 

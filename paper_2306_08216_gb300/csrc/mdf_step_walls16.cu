@@ -12,14 +12,14 @@ cudaError_t walls_batch_occupancy16(int metric, int power_law, int storage, int 
     MDF_WALLS_DISPATCH_ST(kWallsBatchNT, STORAGE_FP16, batch_occupancy_t, occ, smem)
 }
 
-cudaError_t walls_batch_launch16(const BatchItem *items, int nitems, const StepArgs *args, const CUtensorMap *maps,
+cudaError_t walls_batch_launch16(const BatchItem *items, int nitems, int *queue, const StepArgs *args, const CUtensorMap *maps,
                                  int metric, int power_law, int grid, int forced, int roll, int storage,
                                  cudaStream_t stream) {
     if (storage == STORAGE_BF16) {
-        MDF_WALLS_DISPATCH_ST(kWallsBatchNT, STORAGE_BF16, batch_launch_t, items, nitems, args, maps, grid, forced,
+        MDF_WALLS_DISPATCH_ST(kWallsBatchNT, STORAGE_BF16, batch_launch_t, items, nitems, queue, args, maps, grid, forced,
                               roll, stream)
     }
-    MDF_WALLS_DISPATCH_ST(kWallsBatchNT, STORAGE_FP16, batch_launch_t, items, nitems, args, maps, grid, forced, roll,
+    MDF_WALLS_DISPATCH_ST(kWallsBatchNT, STORAGE_FP16, batch_launch_t, items, nitems, queue, args, maps, grid, forced, roll,
                           stream)
 }
 

@@ -812,21 +812,20 @@ __global__ void __launch_bounds__(NT, walls_min_blocks<NT>())
     march_window<NT, MK, PL, FORCED>(&tmap, a, blockIdx.x, blockIdx.y, smem, s_abort);
 }
 
-// Persistent batch form: block b takes work items b, b + gridDim.x, ...
+// Persistent batch form (each_item).
 // FORCED if any problem of the batch has a force, force rate or source;
 // ROLL selects the rolled march, ST the storage mode (see march_walls).
 template <int NT, int MK, bool PL, bool FORCED, bool ROLL, int ST>
 __global__ void __launch_bounds__(NT, kWallsBatchBlocks)
-    walls_batch_kernel(const BatchItem *__restrict__ items, int nitems, const StepArgs *__restrict__ args,
+    walls_batch_kernel(const BatchItem *__restrict__ items, int nitems, int *queue, const StepArgs *__restrict__ args,
                        const CUtensorMap *__restrict__ maps) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ volatile int s_abort[2];
-    for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
-        const BatchItem item = items[w];
+    each_item(items, nitems, queue, [&](const BatchItem &item) {
         march_walls<NT, MK, PL, FORCED, ROLL, ST>(&maps[item.problem], args[item.problem], item.bx, item.by, smem,
                                                   s_abort);
-        if (s_abort[0] || s_abort[1]) break;
-    }
+        return !(s_abort[0] || s_abort[1]);
+    });
 }
 
 template <int NT, int MK, bool PL, bool FORCED>
@@ -860,7 +859,7 @@ cudaError_t occupancy_t(int *occ, int *smem) {
 }
 
 template <int NT, int MK, bool PL, bool FORCED, bool ROLL, int ST>
-cudaError_t batch_launch_ft(const BatchItem *items, int nitems, const StepArgs *args, const CUtensorMap *maps,
+cudaError_t batch_launch_ft(const BatchItem *items, int nitems, int *queue, const StepArgs *args, const CUtensorMap *maps,
                             int grid, cudaStream_t stream) {
     auto k = walls_batch_kernel<NT, MK, PL, FORCED, ROLL, ST>;
     constexpr int smem = walls_smem<NT, FORCED, ST>();
@@ -870,7 +869,7 @@ cudaError_t batch_launch_ft(const BatchItem *items, int nitems, const StepArgs *
         if (e != cudaSuccess) return e;
         mark_device_setup(configured);
     }
-    k<<<grid, NT, smem, stream>>>(items, nitems, args, maps);
+    k<<<grid, NT, smem, stream>>>(items, nitems, queue, args, maps);
     return cudaGetLastError();
 }
 
@@ -883,18 +882,18 @@ constexpr bool walls_unrolled_batch() {
 }
 
 template <int NT, int MK, bool PL, int ST>
-cudaError_t batch_launch_t(const BatchItem *items, int nitems, const StepArgs *args, const CUtensorMap *maps, int grid,
+cudaError_t batch_launch_t(const BatchItem *items, int nitems, int *queue, const StepArgs *args, const CUtensorMap *maps, int grid,
                            int forced, int roll, cudaStream_t stream) {
     if constexpr (walls_unrolled_batch<ST>()) {
         if (!roll) {
-            if (forced) return batch_launch_ft<NT, MK, PL, true, false, ST>(items, nitems, args, maps, grid, stream);
-            return batch_launch_ft<NT, MK, PL, false, false, ST>(items, nitems, args, maps, grid, stream);
+            if (forced) return batch_launch_ft<NT, MK, PL, true, false, ST>(items, nitems, queue, args, maps, grid, stream);
+            return batch_launch_ft<NT, MK, PL, false, false, ST>(items, nitems, queue, args, maps, grid, stream);
         }
     } else {
         if (!roll) return cudaErrorInvalidConfiguration;
     }
-    if (forced) return batch_launch_ft<NT, MK, PL, true, true, ST>(items, nitems, args, maps, grid, stream);
-    return batch_launch_ft<NT, MK, PL, false, true, ST>(items, nitems, args, maps, grid, stream);
+    if (forced) return batch_launch_ft<NT, MK, PL, true, true, ST>(items, nitems, queue, args, maps, grid, stream);
+    return batch_launch_ft<NT, MK, PL, false, true, ST>(items, nitems, queue, args, maps, grid, stream);
 }
 
 // Occupancy of one batch kernel variant.
