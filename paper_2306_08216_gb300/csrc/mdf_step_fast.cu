@@ -56,9 +56,9 @@ constexpr int RHO0_NT = 128;
 // that as many blocks fit an SM as without a force.
 constexpr int FORCE_ROWS = 8;
 
-template <bool FORCED, int ST, bool RHO0>
+template <int FORCE, int ST, bool RHO0>
 __host__ __device__ constexpr int fast_slots() {
-    if (FORCED) return ST == STORAGE_FP32 ? 2 : 3;
+    if (FORCE == FORCE_ANY) return ST == STORAGE_FP32 ? 2 : 3;
     return RHO0 ? FAST_SLOTS_RHO0 : FAST_SLOTS;
 }
 
@@ -96,10 +96,10 @@ __device__ __forceinline__ int row_before(int p, int back, int ny) {
     return r < 0 ? r + ny : r;
 }
 
-template <int NT, int MK, bool FORCED, int ST, bool RHO0>
+template <int NT, int MK, int FORCE, int ST, bool RHO0>
 __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
     fast_kernel(const __grid_constant__ CUtensorMap tmap, const StepArgs a) {
-    constexpr int SLOTS = fast_slots<FORCED, ST, RHO0>();
+    constexpr int SLOTS = fast_slots<FORCE, ST, RHO0>();
     // one TMA row: 10 FP32 planes (15 with alpha = 0), or u, v, P and 4
     // planes of 16-bit pairs
     constexpr int TROW = (RHO0 ? RHO0_PLANES : ST == STORAGE_FP32 ? NPLANES : DEV_PLANES) * NT * 4;
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
     unsigned char *xB00 = ringP0 + RING * P0ROW;
     unsigned char *xF00 = xB00 + 2 * X0ROW;
     uint64_t *mbar = reinterpret_cast<uint64_t *>(xF00 + 2 * X0ROW);
-    unsigned char *ringF = reinterpret_cast<unsigned char *>(mbar + SLOTS);  // force field rows (FORCED)
+    unsigned char *ringF = reinterpret_cast<unsigned char *>(mbar + SLOTS);  // force field rows (FORCE_ANY)
     // one flag per row parity: it is read after the barrier of its row, and a
     // thread can set it again only two barriers later (a plain barrier and a
     // load; with a voting barrier and the row index taken modulo ny by the
@@ -131,7 +131,8 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
     const int nIt = (y1 - y0) + 9;
     const int rowBase = y0 - 4;
     const float c = a.c, inv2c = a.inv2c;
-    constexpr bool forced = FORCED;
+    constexpr bool forced = FORCE != FORCE_NONE;
+    constexpr bool sourced = FORCE == FORCE_ANY;  // a mass source is possible
 
     if (t == 0) {
         s_abort[0] = s_abort[1] = 0;
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
     // body force: F of this column for rows rp + 0, 1 (field), then two rows
     // ahead of every row; the dt step reads the same rows unless a force rate
     // gave it planes of its own
-    const bool ffield = FORCED && a.force_mode == 2;
+    const bool ffield = FORCE == FORCE_ANY && a.force_mode == 2;
     const bool fd_same = ffield && a.force_mode_d == 2 && a.Fxdp == a.Fxp && a.Fydp == a.Fyp;
     int frow = rp;  // the next force row to copy
     auto force_slot = [&](int it) { return ringF + ((it & (FORCE_ROWS - 1)) * 2 * NT + t) * 4; };
@@ -182,10 +183,10 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
     auto force_dt = [&](int it, int r, F2 factor) {
         if (a.force_mode_d == 0) return splat(0.0f);
         if (fd_same) return factor * force_ring(it);
-        if (a.force_mode_d == 1) return factor * mk2(a.Fxd, a.Fyd);
+        if (FORCE == FORCE_CONST || a.force_mode_d == 1) return factor * mk2(a.Fxd, a.Fyd);
         return factor * field_pair(a, a.Fxdp, a.Fydp, (long long)r * a.pitch + GHOST + X);
     };
-    if (FORCED) {
+    if (FORCE == FORCE_ANY) {
         copy_force(0);
         copy_force(1);
     }
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
         constexpr int k = decltype(kc)::value;
         constexpr int s1 = (k + 4) % 5, s2 = (k + 3) % 5, s3 = (k + 2) % 5, s4 = (k + 1) % 5;
         {
-            if (FORCED) {
+            if (FORCE == FORCE_ANY) {
                 copy_force(it + 2);
                 cp_async_wait<2>();  // the copies of row p have landed
             }
@@ -274,7 +275,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
                     float out0[5];
 #pragma unroll
                     for (int j = 0; j < 5; ++j) out0[j] = lds1(P0r, (j * NT + t) * 4);
-                    if (forced && a.r_mode) {
+                    if (sourced && a.r_mode) {
                         const float sR = dw0 * source_at(a, r, X);
 #pragma unroll
                         for (int j = 0; j < 5; ++j) out0[j] += sR;
@@ -300,7 +301,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
                 if (ST == STORAGE_FP32) {
 #pragma unroll
                     for (int j = 0; j < 5; ++j) g[j] = mk2(src[j * NT + t], src[(5 + j) * NT + t]);
-                    const Mom2 m = (forced && a.r_mode)
+                    const Mom2 m = (sourced && a.r_mode)
                                        ? moments2r(g, c, a.rk_hat * source_at(a, rp, X))
                                        : moments2(g, c);
                     noneq2(g, m, inv2c, n);
@@ -392,7 +393,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
                 if (RHO0) {
                     // the same on alpha = 0, with h w_j R
                     float b01 = own01, b03 = own03;
-                    if (forced && a.r_mode) {
+                    if (sourced && a.r_mode) {
                         const float sR = hw0 * source_at(a, rp, X);
                         D0[k][0] += sR;
                         b01 += sR;
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
                     fb[2] = stream2<false>(by2, BY[s1][0], BY[s2][0], BY[s3][0], BY[s4][0], false, wy.w1, wy.w0, wy.w2);
                     fb[4] = stream2<false>(by4, BY[s3][1], BY[s2][1], BY[s1][1], BY[k][1], false, wy.w1, wy.w0, wy.w2);
                     // Step 3: f = feq + (I + h/2 Lt)^-1 (fbar - feq)
-                    const Mom2 m = (forced && a.r_mode) ? moments2r(fb, c, a.rk_bar * source_at(a, qw, X))
+                    const Mom2 m = (sourced && a.r_mode) ? moments2r(fb, c, a.rk_bar * source_at(a, qw, X))
                                                         : moments2(fb, c);
                     F2 n[5], f[5];
                     noneq2(fb, m, inv2c, n);
@@ -434,7 +435,7 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
                     if (RHO0) {
                         // Steps 2-3 on alpha = 0, recovered with u, v of the alpha = 1, 2 fbar
                         float by02 = BY0[s2][0], by04 = BY0[s2][1];
-                        if (forced && a.r_mode) {
+                        if (sourced && a.r_mode) {
                             const float sRq = hw0 * source_at(a, qw, X);
                             by02 += sRq;
                             by04 += sRq;
@@ -488,18 +489,18 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
     }
 }
 
-template <int NT, bool FORCED, int ST, bool RHO0>
+template <int NT, int FORCE, int ST, bool RHO0>
 constexpr int fast_smem() {
-    return fast_slots<FORCED, ST, RHO0>() * (RHO0 ? RHO0_PLANES : ST == STORAGE_FP32 ? NPLANES : DEV_PLANES) * NT * 4 +
+    return fast_slots<FORCE, ST, RHO0>() * (RHO0 ? RHO0_PLANES : ST == STORAGE_FP32 ? NPLANES : DEV_PLANES) * NT * 4 +
            RING * 5 * NT * 8 + 4 * (2 * NT * 8) + (RHO0 ? RING * 5 * NT * 4 + 4 * (2 * NT * 4) : 0) +
-           fast_slots<FORCED, ST, RHO0>() * 8 + (FORCED ? FORCE_ROWS * 2 * NT * 4 : 0);
+           fast_slots<FORCE, ST, RHO0>() * 8 + (FORCE == FORCE_ANY ? FORCE_ROWS * 2 * NT * 4 : 0);
 }
 
-template <int NT, int MK, bool FORCED, int ST, bool RHO0>
+template <int NT, int MK, int FORCE, int ST, bool RHO0>
 cudaError_t fast_launch_t(const CUtensorMap *tmap, const StepArgs &args,
                           const StepPlan &plan, cudaStream_t stream) {
-    auto k = fast_kernel<NT, MK, FORCED, ST, RHO0>;
-    constexpr int smem = fast_smem<NT, FORCED, ST, RHO0>();
+    auto k = fast_kernel<NT, MK, FORCE, ST, RHO0>;
+    constexpr int smem = fast_smem<NT, FORCE, ST, RHO0>();
     static std::atomic<unsigned long long> configured{0};  // devices set up
     if (needs_device_setup(configured)) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -512,29 +513,34 @@ cudaError_t fast_launch_t(const CUtensorMap *tmap, const StepArgs &args,
 
 template <int NT, int MK, int ST, bool RHO0>
 cudaError_t fast_occupancy_t(int *occ, int *smem) {
-    // the variant with a force trades TMA slots for force rows; report the
-    // larger shared memory and the smaller occupancy of the two
-    int o1 = 0, o2 = 0;
-    constexpr int s1 = fast_smem<NT, false, ST, RHO0>(), s2 = fast_smem<NT, true, ST, RHO0>();
-    *smem = s1 > s2 ? s1 : s2;
-    cudaError_t e = cudaFuncSetAttribute(fast_kernel<NT, MK, false, ST, RHO0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, s1);
+    // the variant with force fields trades TMA slots for force rows; report the
+    // largest shared memory and the smallest occupancy of the three
+    *occ = 1 << 30;
+    *smem = 0;
+    const auto variant = [&](auto k, int bytes) {
+        int o = 0;
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, NT, bytes);
+        *occ = std::min(*occ, o);
+        *smem = std::max(*smem, bytes);
+        return e;
+    };
+    cudaError_t e = variant(fast_kernel<NT, MK, FORCE_NONE, ST, RHO0>, fast_smem<NT, FORCE_NONE, ST, RHO0>());
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fast_kernel<NT, MK, true, ST, RHO0>, cudaFuncAttributeMaxDynamicSharedMemorySize, s2);
+        e = variant(fast_kernel<NT, MK, FORCE_CONST, ST, RHO0>, fast_smem<NT, FORCE_CONST, ST, RHO0>());
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, fast_kernel<NT, MK, false, ST, RHO0>, NT, s1);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, fast_kernel<NT, MK, true, ST, RHO0>, NT, s2);
-    *occ = o1 < o2 ? o1 : o2;
+        e = variant(fast_kernel<NT, MK, FORCE_ANY, ST, RHO0>, fast_smem<NT, FORCE_ANY, ST, RHO0>());
     return e;
 }
 
 template <int NT, int MK, int ST, bool RHO0>
 cudaError_t fast_launch_f(const CUtensorMap *tmap, const StepArgs &args,
                           const StepPlan &plan, cudaStream_t stream) {
-    return (args.force_mode || args.force_mode_d || args.r_mode)
-               ? fast_launch_t<NT, MK, true, ST, RHO0>(tmap, args, plan, stream)
-               : fast_launch_t<NT, MK, false, ST, RHO0>(tmap, args, plan, stream);
+    switch (force_kind(args)) {
+        case FORCE_NONE: return fast_launch_t<NT, MK, FORCE_NONE, ST, RHO0>(tmap, args, plan, stream);
+        case FORCE_CONST: return fast_launch_t<NT, MK, FORCE_CONST, ST, RHO0>(tmap, args, plan, stream);
+        default: return fast_launch_t<NT, MK, FORCE_ANY, ST, RHO0>(tmap, args, plan, stream);
+    }
 }
 
 template <int NT, int MK>

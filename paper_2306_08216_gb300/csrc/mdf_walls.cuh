@@ -469,10 +469,10 @@ __device__ __forceinline__ void march_walls(const CUtensorMap *tmap, const StepA
 // march_walls; stretched 1200 x 700 channel 35 against 38).  On a full GPU, in
 // the batches, march_walls is the faster (512 power-law cavities 1.81 -> 1.57 ms a
 // step).
-template <int NT, int MK, bool PL, bool FORCED>
+template <int NT, int MK, bool PL, int FORCE>
 __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const StepArgs &a, int bx, int by,
                                              unsigned char *smem, volatile int *s_abort) {
-    constexpr int SLOTS = walls_slots<NT, FORCED>();
+    constexpr int SLOTS = walls_slots<NT, FORCE == FORCE_ANY>();
     constexpr int TROW = NPLANES * NT * 4;  // one TMA row
     constexpr int PROW = 5 * NT * 8;        // one fhat^+ ring row
     constexpr int XROW = 2 * NT * 8;        // one exchange row: pops 1, 3
@@ -482,7 +482,7 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
     unsigned char *xF0 = xB0 + 2 * XROW;       // f(t+h) of pops 1, 3 of row q (two buffers)
     unsigned char *nrow = xF0 + 2 * XROW;      // f(t+h) of pops 2, 4 of the north wall row
     uint64_t *mbar = reinterpret_cast<uint64_t *>(nrow + 2 * NT * 8);
-    unsigned char *ringF = reinterpret_cast<unsigned char *>(mbar + SLOTS);  // force field rows (FORCED)
+    unsigned char *ringF = reinterpret_cast<unsigned char *>(mbar + SLOTS);  // force field rows (FORCE_ANY)
 
     const int t = threadIdx.x;
     const int x0 = bx * a.W;
@@ -522,7 +522,7 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
 
     // body force (fields): F of this column two rows ahead of every row; the dt
     // step reads the same rows unless a force rate gave it planes of its own
-    const bool ffield = FORCED && a.force_mode == 2;
+    const bool ffield = FORCE == FORCE_ANY && a.force_mode == 2;
     const bool fd_same = ffield && a.force_mode_d == 2 && a.Fxdp == a.Fxp && a.Fydp == a.Fyp;
     int frow = rp;
     auto force_slot = [&](int it) { return ringF + ((it & (WALL_FORCE_ROWS - 1)) * 2 * NT + t) * 4; };
@@ -550,11 +550,11 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
     auto force_dt = [&](int it, int row, F2 factor) {
         if (a.force_mode_d == 0) return splat(0.0f);
         if (fd_same) return factor * force_ring(it);
-        if (a.force_mode_d == 1) return factor * mk2(a.Fxd, a.Fyd);
+        if (FORCE == FORCE_CONST || a.force_mode_d == 1) return factor * mk2(a.Fxd, a.Fyd);
         if (!col_in) return splat(0.0f);
         return factor * field_pair(a, a.Fxdp, a.Fydp, (long long)row * a.pitch + GHOST + X);
     };
-    if (FORCED) {
+    if (FORCE == FORCE_ANY) {
         copy_force(0);
         copy_force(1);
     }
@@ -593,7 +593,7 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
         constexpr int k = decltype(kc)::value;
         constexpr int s1 = (k + 4) % 5, s2 = (k + 3) % 5, s3 = (k + 2) % 5, s4 = (k + 1) % 5;
         {
-            if (FORCED) {
+            if (FORCE == FORCE_ANY) {
                 copy_force(it + 2);
                 cp_async_wait<2>();  // the copies of row p have landed
             }
@@ -608,7 +608,7 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
                     F2 out[5];
 #pragma unroll
                     for (int j = 0; j < 5; ++j) out[j] = lds2(Pr, (j * NT + t) * 8);
-                    if (FORCED) {
+                    if (FORCE != FORCE_NONE) {
                         const F2 fF = force_dt(it - 5, r, pair_of(a.pdw));
 #pragma unroll
                         for (int j = 0; j < 5; ++j) out[j] = out[j] + fF;
@@ -648,7 +648,7 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
                 F2 g[5], n[5], o[5];
 #pragma unroll
                 for (int j = 0; j < 5; ++j) g[j] = mk2(src[j * NT + t], src[(5 + j) * NT + t]);
-                const Mom2 m = (FORCED && a.r_mode && p_in && col_in)
+                const Mom2 m = (FORCE == FORCE_ANY && a.r_mode && p_in && col_in)
                                    ? moments2r(g, c, a.rk_hat * source_at(a, rp, X))
                                    : moments2(g, c);
                 noneq2(g, m, inv2c, n);
@@ -703,7 +703,7 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
             if (calc) {
                 // pass 1, x part of row p
                 F2 hF = zero;
-                if (FORCED && p_in) hF = force_h(it, pair_of(a.phw));
+                if (FORCE != FORCE_NONE && p_in) hF = force_h(it, pair_of(a.phw));
                 D013[k][0] = D013[k][0] + hF;
                 D013[k][1] = stream2<true>(own1 + hF, lds2(xB, (t + 1) * 8), own1, lds2(xB, (t - 1) * 8),
                                            lds2(xB, (t - 2) * 8), xadj_p, wxh.w1, wxh.w0, wxh.w2);
@@ -717,7 +717,7 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
                         FY[s2][1] = lds2(nrow, (NT + t) * 8);
                     } else if (!(ywall && q == 0)) {
                         F2 hFq = zero;
-                        if (FORCED) hFq = force_h(it - 2, pair_of(a.phw));
+                        if (FORCE != FORCE_NONE) hFq = force_h(it - 2, pair_of(a.phw));
                         W3 wy;
                         if (MK == METRIC_UNIFORM) wy = {pair_of(a.pwyh[0]), pair_of(a.pwyh[1]), pair_of(a.pwyh[2])};
                         else wy = weights(a.kyv[q], a.h, a);
@@ -736,7 +736,7 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
                             mKk = splat(-(1.0f - RK[s2][0]));
                             Dk = splat(0.5f * (RK[s2][1] - RK[s2][0]));
                         }
-                        const Mom2 m = (FORCED && a.r_mode && col_in) ? moments2r(fb, c, a.rk_bar * source_at(a, q, X))
+                        const Mom2 m = (FORCE == FORCE_ANY && a.r_mode && col_in) ? moments2r(fb, c, a.rk_bar * source_at(a, q, X))
                                                             : moments2(fb, c);
                         F2 n[5], f[5];
                         noneq2(fb, m, inv2c, n);
@@ -785,7 +785,7 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
         if (it0 + 4 >= nIt) break;
         if (!row(it0 + 4, integral_constant<int, 4>{}, 4)) { aborted = true; break; }
     }
-    if (FORCED) cp_async_wait<0>();
+    if (FORCE == FORCE_ANY) cp_async_wait<0>();
     if (aborted && t == 0) {
         for (int it = issued - SLOTS; it < issued; ++it) {
             if (it < 0) continue;
@@ -804,12 +804,12 @@ constexpr int walls_min_blocks() {
     return NT <= 128 ? 3 : 2;
 }
 
-template <int NT, int MK, bool PL, bool FORCED>
+template <int NT, int MK, bool PL, int FORCE>
 __global__ void __launch_bounds__(NT, walls_min_blocks<NT>())
     walls_kernel(const __grid_constant__ CUtensorMap tmap, const StepArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ volatile int s_abort[2];
-    march_window<NT, MK, PL, FORCED>(&tmap, a, blockIdx.x, blockIdx.y, smem, s_abort);
+    march_window<NT, MK, PL, FORCE>(&tmap, a, blockIdx.x, blockIdx.y, smem, s_abort);
 }
 
 // Persistent batch form (each_item).
@@ -828,33 +828,37 @@ __global__ void __launch_bounds__(NT, kWallsBatchBlocks)
     });
 }
 
-template <int NT, int MK, bool PL, bool FORCED>
+template <int NT, int MK, bool PL, int FORCE>
 cudaError_t launch_t(const CUtensorMap *tmap, const StepArgs &args, const StepPlan &plan, cudaStream_t stream) {
-    auto k = walls_kernel<NT, MK, PL, FORCED>;
+    auto k = walls_kernel<NT, MK, PL, FORCE>;
+    constexpr int smem = walls_smem<NT, FORCE == FORCE_ANY>();
     static std::atomic<unsigned long long> configured{0};  // devices set up
     if (needs_device_setup(configured)) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (walls_smem<NT, FORCED>()));
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         mark_device_setup(configured);
     }
-    k<<<dim3(plan.gx, plan.gy), NT, walls_smem<NT, FORCED>(), stream>>>(*tmap, args);
+    k<<<dim3(plan.gx, plan.gy), NT, smem, stream>>>(*tmap, args);
     return cudaGetLastError();
 }
 
 template <int NT, int MK, bool PL>
 cudaError_t occupancy_t(int *occ, int *smem) {
-    // the variant with a force holds force rows as well: report the larger
-    // shared memory and the smaller occupancy of the two
-    int o1 = 0, o2 = 0;
-    constexpr int s1 = walls_smem<NT, false>(), s2 = walls_smem<NT, true>();
-    *smem = s1 > s2 ? s1 : s2;
-    cudaError_t e =
-        cudaFuncSetAttribute(walls_kernel<NT, MK, PL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(walls_kernel<NT, MK, PL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, s2);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, walls_kernel<NT, MK, PL, false>, NT, s1);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, walls_kernel<NT, MK, PL, true>, NT, s2);
-    *occ = o1 < o2 ? o1 : o2;
+    // the variant with force fields holds force rows as well: report the largest
+    // shared memory and the smallest occupancy of the three
+    *occ = 1 << 30;
+    *smem = 0;
+    const auto variant = [&](auto k, int bytes) {
+        int o = 0;
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, NT, bytes);
+        *occ = std::min(*occ, o);
+        *smem = std::max(*smem, bytes);
+        return e;
+    };
+    cudaError_t e = variant(walls_kernel<NT, MK, PL, FORCE_NONE>, walls_smem<NT, false>());
+    if (e == cudaSuccess) e = variant(walls_kernel<NT, MK, PL, FORCE_CONST>, walls_smem<NT, false>());
+    if (e == cudaSuccess) e = variant(walls_kernel<NT, MK, PL, FORCE_ANY>, walls_smem<NT, true>());
     return e;
 }
 
@@ -940,8 +944,11 @@ cudaError_t batch_occupancy_t(int *occ, int *smem) {
 
 template <int NT, int MK, bool PL>
 cudaError_t launch_f(const CUtensorMap *tmap, const StepArgs &args, const StepPlan &plan, cudaStream_t stream) {
-    if (args.force_mode || args.force_mode_d || args.r_mode) return launch_t<NT, MK, PL, true>(tmap, args, plan, stream);
-    return launch_t<NT, MK, PL, false>(tmap, args, plan, stream);
+    switch (force_kind(args)) {
+        case FORCE_NONE: return launch_t<NT, MK, PL, FORCE_NONE>(tmap, args, plan, stream);
+        case FORCE_CONST: return launch_t<NT, MK, PL, FORCE_CONST>(tmap, args, plan, stream);
+        default: return launch_t<NT, MK, PL, FORCE_ANY>(tmap, args, plan, stream);
+    }
 }
 
 template <int NT>
