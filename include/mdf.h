@@ -304,9 +304,9 @@ mdf_status mdf_launch_info(const mdf_ctx *ctx, int info[8]);
  * band of `rows_per_block` (>= 1) rows, and the tile kernel (threads = 0;
  * rows_per_block 8 picks tiles of 8 x 8 nodes where the grid is small enough
  * to have that plan, anything else 16 x 16; the values are the same), where a
- * block of 256 threads computes one tile in three phases with a recomputed
- * halo of 4 nodes: on grids too small to fill the GPU with long bands it
- * avoids the serial march
+ * block of 256 or 288 threads computes one tile in three phases with a
+ * recomputed halo of 4 nodes: on grids too small to fill the GPU with long
+ * bands it avoids the serial march
  * (every storage mode, not with the alpha = 0 distribution; the only plan
  * for 16-bit storage off the periodic fast path).  mdf_create times every
  * candidate plan for a few steps and keeps the fastest (the tile kernel only

@@ -104,7 +104,7 @@ int step_candidates(int metric, int power_law, int walls, int storage, int rho0,
             const auto tile_plan = [&](int tw, int th) {
                 StepPlan &p = out[n++];
                 p.kind = PLAN_TILE;
-                p.NT = tx * ty;
+                p.NT = tile_threads(tw, storage, rho0 != 0);
                 p.W = tw;
                 p.H = th;
                 p.gx = (nx + tw - 1) / tw;
@@ -117,7 +117,8 @@ int step_candidates(int metric, int power_law, int walls, int storage, int rho0,
             // blocks each: from about there on their larger halo costs more than
             // the shorter phases give
             const long long small = (long long)((nx + 7) / 8) * ((ny + 7) / 8);
-            if (storage == STORAGE_FP32 && !rho0 && n < max && small <= 3ll * (num_sms > 0 ? num_sms : 1)) tile_plan(8, 8);
+            if (storage == STORAGE_FP32 && !rho0 && n < max && small <= 3ll * (num_sms > 0 ? num_sms : 1))
+                tile_plan(kSmallTile, kSmallTile);
         }
     }
     return n;

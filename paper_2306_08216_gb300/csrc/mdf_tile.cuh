@@ -53,19 +53,8 @@ __device__ __forceinline__ int axis_index(int i, int n, bool wall) {
     return wrap(i, n);
 }
 
-// Threads of a block: one per output node on the 16 x 16 tile; on the 8 x 8
-// tile the same 256, one per node of the 16 x 16 region of phase A, so that each
-// phase is a single pass.  The small tile recomputes more (4 and 2.25 times the
-// output in phases A and B, against 2.25 and 1.56), which costs nothing on a
-// grid that leaves most SMs without a block, where the length of a block's three
-// phases is the time of the step (64^2 periodic nodes, 16 -> 64
-// blocks: 3.72 -> 2.56 us a step).
-constexpr int kTileThreads = 256;
-constexpr int kSmallTile = 8;
-
 template <int TX, int TY>
 struct Tile {
-    static constexpr int NT = kTileThreads;
     static constexpr int N0 = TX * TY;  // output nodes
     static constexpr int X8 = TX + 8, Y8 = TY + 8, N8 = X8 * Y8;  // fbar^+ region: tile + 4
     static constexpr int X4 = TX + 4, Y4 = TY + 4, N4 = X4 * Y4;  // f region: tile + 2
@@ -202,6 +191,7 @@ __device__ __forceinline__ void tile_output(const StepArgs &a, int X, int Y, int
 template <int TX, int TY, int MK, bool PL, bool WALLS, int ST, bool RHO0>
 __device__ __forceinline__ void tile_step(const StepArgs &a, int bx, int by, unsigned char *smem) {
     using T = Tile<TX, TY>;
+    constexpr int NT = tile_threads(TX, ST, RHO0);
     unsigned char *Bs = smem;                          // fbar^+ [5][N8] pairs
     unsigned char *Fs = smem + T::B_BYTES;             // f(t+h) [5][N4] pairs
     float *Ks = reinterpret_cast<float *>(Fs + T::F_BYTES);  // power law: rkp [N4], rk [N4]
@@ -220,7 +210,7 @@ __device__ __forceinline__ void tile_step(const StepArgs &a, int bx, int by, uns
     // nodes of the halo ring (4 rows above, 4 below, 4 columns each side).
     // All their loads are issued before any arithmetic, so that the passes
     // share one memory latency.
-    constexpr int PASSES = (T::N8 + T::NT - 1) / T::NT;
+    constexpr int PASSES = (T::N8 + NT - 1) / NT;
     auto region_node = [&](int i, int &lx, int &ly) {
         if (i < T::N0) {
             lx = 4 + i % TX;
@@ -248,7 +238,7 @@ __device__ __forceinline__ void tile_step(const StepArgs &a, int bx, int by, uns
     float raw[PASSES][NW];
 #pragma unroll
     for (int q = 0; q < PASSES; ++q) {
-        const int i = t + q * T::NT;
+        const int i = t + q * NT;
 #pragma unroll
         for (int k = 0; k < NW; ++k) raw[q][k] = 0.0f;
         if (i < T::N8) {
@@ -269,7 +259,7 @@ __device__ __forceinline__ void tile_step(const StepArgs &a, int bx, int by, uns
     float hp0[5];  // ... and of its alpha = 0 populations
 #pragma unroll
     for (int q = 0; q < PASSES; ++q) {
-        const int i = t + q * T::NT;
+        const int i = t + q * NT;
         if (i >= T::N8) break;
         int lx, ly;
         region_node(i, lx, ly);
@@ -344,7 +334,7 @@ __device__ __forceinline__ void tile_step(const StepArgs &a, int bx, int by, uns
     const F2 hw = splat(a.h * 0.2f);
     const F2 mKk = pair_of_bits(a.pmKk), Dk = pair_of_bits(a.pDk);
 #pragma unroll 1
-    for (int i4 = t; i4 < T::N4; i4 += T::NT) {
+    for (int i4 = t; i4 < T::N4; i4 += NT) {
         const int lx4 = i4 % T::X4, ly4 = i4 / T::X4;
         const int X = x0 - 2 + lx4, Y = y0 - 2 + ly4;
         if (WALLS) {
@@ -410,7 +400,7 @@ __device__ __forceinline__ void tile_step(const StepArgs &a, int bx, int by, uns
         // wall nodes of the f region from their interior neighbour (corners:
         // the diagonal neighbour and the west/east wall velocity)
 #pragma unroll 1
-        for (int i4 = t; i4 < T::N4; i4 += T::NT) {
+        for (int i4 = t; i4 < T::N4; i4 += NT) {
             const int lx4 = i4 % T::X4, ly4 = i4 / T::X4;
             const int X = x0 - 2 + lx4, Y = y0 - 2 + ly4;
             const bool inx = X >= 0 && X < a.nx, iny = Y >= 0 && Y < a.ny;
@@ -443,7 +433,7 @@ __device__ __forceinline__ void tile_step(const StepArgs &a, int bx, int by, uns
     // ------------------------------------------------ C: fhat(t+dt) of the own node
     const int li = t % TX, lj = t / TX;
     const int X = x0 + li, Y = y0 + lj;
-    if (T::N0 < T::NT && t >= T::N0) return;
+    if (T::N0 < NT && t >= T::N0) return;
     if (X >= a.nx || Y >= a.ny) return;
     if (WALLS && ((xwall && (X == 0 || X == a.nx - 1)) || (ywall && (Y == 0 || Y == a.ny - 1)))) return;
     tile_output<TX, TY, MK, WALLS, ST, RHO0>(a, X, Y, li, lj, Fs, Fs0, hp, hp0);
@@ -530,7 +520,7 @@ __device__ __forceinline__ void tile_output(const StepArgs &a, int X, int Y, int
 }
 
 template <int TX, int TY, int MK, bool PL, bool WALLS, int ST, bool RHO0>
-__global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) tile_kernel(const StepArgs a) {
+__global__ void __launch_bounds__(tile_threads(TX, ST, RHO0), kTileMinBlocks) tile_kernel(const StepArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     // launched with programmatic stream serialization: the block touches
     // global memory only after the previous step has completed.  The next
@@ -544,7 +534,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) tile_kernel(cons
 // Many problems in one persistent launch: block b steps work items
 // b, b + gridDim.x, ... (problem, tile x, tile y), largest problems first.
 template <int TX, int TY, int MK, bool PL, bool WALLS, int ST>
-__global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) tile_batch_kernel(const BatchItem *__restrict__ items, int nitems,
+__global__ void __launch_bounds__(tile_threads(TX, ST, false), kTileMinBlocks) tile_batch_kernel(const BatchItem *__restrict__ items, int nitems,
                                                                const StepArgs *__restrict__ args) {
     extern __shared__ __align__(128) unsigned char smem[];
     for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
@@ -567,7 +557,7 @@ cudaError_t tile_occupancy_t(int *occ, int *smem) {
     *smem = tile_smem<MK, PL, WALLS, RHO0>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, kTileThreads, *smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, tile_threads(kTX, ST, RHO0), *smem);
 }
 
 // One step with tiles of TS x TS nodes.
@@ -585,7 +575,7 @@ cudaError_t tile_launch_ts(const StepArgs &args, const StepPlan &plan, cudaStrea
     // scheduled while this one drains (tile_kernel waits for it in hardware)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(plan.gx, plan.gy);
-    cfg.blockDim = dim3(kTileThreads);
+    cfg.blockDim = dim3(tile_threads(TS, ST, RHO0));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -614,7 +604,7 @@ cudaError_t tile_batch_occupancy_t(int *occ, int *smem) {
     *smem = tile_smem<MK, PL, WALLS>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, kTileThreads, *smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, tile_threads(kTX, ST, false), *smem);
 }
 
 template <int MK, bool PL, bool WALLS, int ST>
@@ -627,7 +617,7 @@ cudaError_t tile_batch_launch_t(const BatchItem *items, int nitems, const StepAr
         if (e != cudaSuccess) return e;
         mark_device_setup(configured);
     }
-    k<<<grid, kTileThreads, tile_smem<MK, PL, WALLS>(), stream>>>(items, nitems, args);
+    k<<<grid, tile_threads(kTX, ST, false), tile_smem<MK, PL, WALLS>(), stream>>>(items, nitems, args);
     return cudaGetLastError();
 }
 
