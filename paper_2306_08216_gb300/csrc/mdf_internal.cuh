@@ -143,13 +143,13 @@ constexpr int TILE_X = 16, TILE_Y = 16;  // output tile of the tile kernel (halo
 // Threads of a block.  16 x 16 tiles: 288, so that the 24 x 24 nodes of phase A
 // are two full passes (with one thread per output node the third pass had work
 // for two warps of eight, and the block waited for them: power-law trapezoid of
-// 513^2 1177 -> 1087 us for 50 steps, 300^2 power-law cavity 8.8 -> 8.5 us a step); the 16-bit modes
-// and the alpha = 0 lane, whose registers that would spill, 256.  8 x 8 tiles:
-// 256, one per node of their 16 x 16 region, so that each phase is a single pass.
-// The small tile recomputes more (4 and 2.25 times the output in phases A and B,
-// against 2.25 and 1.56), which costs nothing on a grid that leaves most SMs
-// without a block, where the length of a block's three phases is the time of the
-// step (64^2 periodic nodes, 16 -> 64 blocks: 3.72 -> 2.56 us a step).
+// 513^2 24.5 -> 22.7 us a step, 300^2 power-law cavity 8.8 -> 8.5); the 16-bit
+// modes and the alpha = 0 lane, whose registers that would spill, 256.  8 x 8
+// tiles: 256, one per node of their 16 x 16 region, so that each phase is a single
+// pass.  The small tile recomputes more (4 and 2.25 times the output in phases A
+// and B, against 2.25 and 1.56), which costs nothing on a grid that leaves most
+// SMs without a block, where the length of a block's three phases is the time of
+// the step (64^2 periodic nodes, 16 -> 64 blocks: 3.72 -> 2.56 us a step).
 constexpr int kSmallTile = 8;
 constexpr int tile_threads(int ts, int storage, bool rho0) {
     return ts != kSmallTile && storage == STORAGE_FP32 && !rho0 ? 288 : 256;
