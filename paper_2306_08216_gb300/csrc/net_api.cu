@@ -287,7 +287,19 @@ static mdf_status backward(mdf_net *n, int B) {
     NCK(n, pool_backward(n->dp0, n->dz[12], n->z[1], n->dz[1], B, R, 32, n->stream));
     NRET(wgrad(n, 1, B, n->dz[1], n->y[0]));
     NRET(back(n, 1, B));
-    return wgrad(n, 0, B, n->dz[0], n->xin);
+    NRET(wgrad(n, 0, B, n->dz[0], n->xin));
+    // every dz is still in place
+    BiasArgs a;
+    a.layers = kNL;
+    for (int l = 0; l < kNL; ++l) {
+        a.P[l] = pix(n, B, kLayers[l].div);
+        a.cout_real[l] = kLayers[l].cout;
+        a.cout_pad[l] = n->cout_pad[l];
+        a.dZ[l] = n->dz[l];
+        a.g[l] = n->grad + n->off[l] + (long long)kLayers[l].cout * 9 * kLayers[l].cin;
+    }
+    NCK(n, bias_grads(a, n->stream));
+    return MDF_OK;
 }
 
 // Wait for the stream; a tensor-core kernel that gave up waiting for its

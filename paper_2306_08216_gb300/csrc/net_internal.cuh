@@ -62,10 +62,10 @@ cudaError_t conv_forward(const ConvArgs &a, cudaStream_t st);
 bool conv_tc_applies(const ConvArgs &a);
 cudaError_t conv_forward_tc(const ConvArgs &a, int num_sms, int *err, cudaStream_t st);
 
-// Weight and bias gradients of one layer, accumulated (atomic FP32) into the
-// flat parameter-gradient vector: g[off + (co * 9 + tap) * cin_real + ci]
+// Weight gradient of one layer, accumulated (atomic FP32) into the flat
+// parameter-gradient vector: g[off + (co * 9 + tap) * cin_real + ci]
 // += sum_m dZ[m][co] X[m shifted by tap][ci] for co < cout_real,
-// ci < cin_real, and g[off + cout_real * 9 * cin_real + co] += sum_m dZ[m][co].
+// ci < cin_real.
 struct WGradArgs {
     const bf16 *dZ;  // [B][R][R][Cout]
     const bf16 *X;   // [B][R][R][Cin]
@@ -73,12 +73,34 @@ struct WGradArgs {
     long long off;
     int B, R, Cin, Cout, cin_real, cout_real;
 };
+// How the pixels are split: `splits` runs of `chunk` pieces of 32 pixels (the last
+// run may be shorter), one FP32 chain and one atomic addition per run.  Enough
+// blocks of the mma.sync kernel to put four on every SM.
+struct WGradSplit {
+    long long ktiles, chunk, splits;
+};
+WGradSplit wgrad_split(const WGradArgs &a, int num_sms);
 cudaError_t conv_wgrad(const WGradArgs &a, int num_sms, cudaStream_t st);
-// The same sums on the tcgen05 tensor cores (net_wgrad.cu).  Applies when R is
-// a power of two of at least 8, Cin is 32 or a multiple of 64 and Cout 32, 64
-// or a multiple of 128; a CTA that gives up waiting sets *err (device memory).
+// The same sums on the tcgen05 tensor cores (net_wgrad.cu), run by run equal to
+// the bit.  Applies when R is a power of two of at least 8, Cin is 32 or a
+// multiple of 64 and Cout 32, 64 or a multiple of 128; a CTA that gives up
+// waiting sets *err (device memory).
 bool conv_wgrad_tc_applies(const WGradArgs &a);
 cudaError_t conv_wgrad_tc(const WGradArgs &a, int num_sms, int *err, cudaStream_t st);
+
+constexpr int kMaxLayers = 16;
+
+// Bias gradients of every layer, accumulated (atomic FP32): g[l][co] +=
+// sum_m dZ[l][m][co] for co < cout_real[l], m < P[l].
+struct BiasArgs {
+    int layers;
+    long long first[kMaxLayers + 1];  // set by bias_grads
+    long long P[kMaxLayers];
+    int cout_real[kMaxLayers], cout_pad[kMaxLayers];
+    const bf16 *dZ[kMaxLayers];
+    float *g[kMaxLayers];
+};
+cudaError_t bias_grads(BiasArgs a, cudaStream_t st);
 
 // Elementwise / layout kernels (n = element count unless stated).
 cudaError_t silu_forward(const bf16 *z, bf16 *y, long long n, cudaStream_t st);
@@ -104,7 +126,6 @@ cudaError_t mse_loss(const float *o, const float *t, bf16 *dout, double *loss, i
 // Layer weights from the flat FP32 parameter vector: forward BF16
 // [cout_pad][9][cin_pad], mirrored BF16 [cin_pad][9][cout_pad] and FP32 bias
 // [cout_pad], zero in the padding; every layer in one launch.
-constexpr int kMaxLayers = 16;
 struct PrepareArgs {
     const float *params;
     int layers;

@@ -219,21 +219,13 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WGradArgs a, int chunk) {
         }
     };
 
-    // The MMAs' FP32 accumulation drops low bits at every step: chains of at
-    // most 16 of them (8 K tiles), with rounded additions in between.
-    float acc[2][4][4], sum[2][4][4];
-    auto flush = [&](bool first) {
+    float acc[2][4][4];
 #pragma unroll
-        for (int mi = 0; mi < 2; ++mi)
+    for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
-            for (int ni = 0; ni < 4; ++ni)
+        for (int ni = 0; ni < 4; ++ni)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    sum[mi][ni][e] = first ? 0.0f : sum[mi][ni][e] + acc[mi][ni][e];
-                    acc[mi][ni][e] = 0.0f;
-                }
-    };
-    flush(true);
+            for (int e = 0; e < 4; ++e) acc[mi][ni][e] = 0.0f;
 
     load(kt0);
     store(0);
@@ -243,10 +235,8 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WGradArgs a, int chunk) {
         if (kt + 1 < kt1) load(kt + 1);
         warp_tile_k32(As[cur], Bs[cur], wm * 32, wn * 32, lane, acc);
         if (kt + 1 < kt1) store(cur ^ 1);
-        if (((kt - kt0) & 7) == 7) flush(false);
         __syncthreads();
     }
-    flush(false);
 
     const int g = lane >> 2, c = lane & 3;
 #pragma unroll
@@ -260,18 +250,49 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WGradArgs a, int chunk) {
                 if (co >= a.cout_real || n >= NC) continue;
                 const int tap = n / a.Cin, ci = n - tap * a.Cin;
                 if (ci >= a.cin_real) continue;
-                atomicAdd(a.g + a.off + ((long long)co * 9 + tap) * a.cin_real + ci, sum[mi][ni][e]);
+                atomicAdd(a.g + a.off + ((long long)co * 9 + tap) * a.cin_real + ci, acc[mi][ni][e]);
             }
 }
 
-// Bias gradient: sum over pixels of dZ[m][co], one block per pixel chunk.
-__global__ void bias_grad_kernel(const bf16 *dZ, long long P, int Cout, int cout_real, long long chunk, float *g) {
-    const long long p0 = (long long)blockIdx.x * chunk;
-    const long long p1 = p0 + chunk < P ? p0 + chunk : P;
-    for (int co = threadIdx.x; co < cout_real; co += blockDim.x) {
-        float s = 0.0f;
-        for (long long p = p0; p < p1; ++p) s += __bfloat162float(dZ[p * Cout + co]);
-        atomicAdd(g + co, s);
+// Bias gradient g[co] += sum over pixels of dZ[m][co], every layer in one launch.
+// Work item = two channels of a run of 256 pixels, summed in the order of the
+// pixels (one FP32 chain, one atomic addition): the order is part of the result,
+// so a run is not split further.  The loads of 32 pixels are issued ahead of their
+// additions.  Bound: reading dZ once, from HBM for the most part (16 samples of
+// 128 x 128: 39 us for 15 layers; a launch per layer, one channel and one load
+// at a time per thread, took 670 us).
+constexpr int BIAS_RUN = 256;
+
+__global__ void __launch_bounds__(128) bias_grad_kernel(const BiasArgs a) {
+    const long long n = a.first[a.layers];
+    for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += (long long)gridDim.x * blockDim.x) {
+        int l = 0;
+        while (w >= a.first[l + 1]) ++l;
+        const long long i = w - a.first[l];
+        const int pairs = (a.cout_real[l] + 1) / 2, co = 2 * (int)(i % pairs), C = a.cout_pad[l];
+        const long long p0 = i / pairs * BIAS_RUN;
+        const int m = (int)(a.P[l] - p0 < BIAS_RUN ? a.P[l] - p0 : BIAS_RUN);
+        const bf16 *z = a.dZ[l] + p0 * C + co;
+        float s0 = 0.0f, s1 = 0.0f;
+        int p = 0;
+        for (; p + 32 <= m; p += 32) {
+            __nv_bfloat162 v[32];
+#pragma unroll
+            for (int k = 0; k < 32; ++k) v[k] = *reinterpret_cast<const __nv_bfloat162 *>(z + (long long)(p + k) * C);
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+                const float2 f = __bfloat1622float2(v[k]);
+                s0 += f.x;
+                s1 += f.y;
+            }
+        }
+        for (; p < m; ++p) {
+            const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(z + (long long)p * C));
+            s0 += f.x;
+            s1 += f.y;
+        }
+        atomicAdd(a.g[l] + co, s0);
+        if (co + 1 < a.cout_real[l]) atomicAdd(a.g[l] + co + 1, s1);
     }
 }
 
@@ -500,22 +521,32 @@ cudaError_t conv_forward(const ConvArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t conv_wgrad(const WGradArgs &a, int num_sms, cudaStream_t st) {
-    if (a.Cin % 8 || a.Cout % 8) return cudaErrorInvalidValue;
-    const long long P = (long long)a.B * a.R * a.R;
-    const long long ktiles = (P + 31) / 32;
+WGradSplit wgrad_split(const WGradArgs &a, int num_sms) {
+    WGradSplit w;
+    w.ktiles = ((long long)a.B * a.R * a.R + 31) / 32;
     const int tn = (9 * a.Cin + WBN - 1) / WBN, tm = (a.Cout + WBM - 1) / WBM;
     long long splits = (4ll * num_sms + tn * tm - 1) / (tn * tm);
-    if (splits > ktiles) splits = ktiles;
+    if (splits > w.ktiles) splits = w.ktiles;
     if (splits < 1) splits = 1;
-    const long long chunk = (ktiles + splits - 1) / splits;
-    splits = (ktiles + chunk - 1) / chunk;
-    wgrad_kernel<<<dim3(tn, tm, (unsigned)splits), 256, 0, st>>>(a, (int)chunk);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const long long pchunk = 256;
-    bias_grad_kernel<<<(unsigned)((P + pchunk - 1) / pchunk), 256, 0, st>>>(
-        a.dZ, P, a.Cout, a.cout_real, pchunk, a.g + a.off + (long long)a.cout_real * 9 * a.cin_real);
+    w.chunk = (w.ktiles + splits - 1) / splits;
+    w.splits = (w.ktiles + w.chunk - 1) / w.chunk;
+    return w;
+}
+
+cudaError_t conv_wgrad(const WGradArgs &a, int num_sms, cudaStream_t st) {
+    if (a.Cin % 8 || a.Cout % 8) return cudaErrorInvalidValue;
+    const int tn = (9 * a.Cin + WBN - 1) / WBN, tm = (a.Cout + WBM - 1) / WBM;
+    const WGradSplit w = wgrad_split(a, num_sms);
+    wgrad_kernel<<<dim3(tn, tm, (unsigned)w.splits), 256, 0, st>>>(a, (int)w.chunk);
+    return cudaGetLastError();
+}
+
+cudaError_t bias_grads(BiasArgs a, cudaStream_t st) {
+    a.first[0] = 0;
+    for (int l = 0; l < a.layers; ++l)
+        a.first[l + 1] = a.first[l] + (a.P[l] + BIAS_RUN - 1) / BIAS_RUN * ((a.cout_real[l] + 1) / 2);
+    const long long blocks = (a.first[a.layers] + 127) / 128;
+    bias_grad_kernel<<<(unsigned)(blocks < (1 << 20) ? blocks : 1 << 20), 128, 0, st>>>(a);
     return cudaGetLastError();
 }
 
