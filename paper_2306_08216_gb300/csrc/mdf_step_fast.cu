@@ -478,6 +478,8 @@ __global__ void __launch_bounds__(NT, RHO0 ? 3 : (NT <= 128 ? 4 : 2))
         if (it0 + 4 >= nIt) break;
         if (!row(it0 + 4, integral_constant<int, 4>{}, 4)) { aborted = true; break; }
     }
+    // an aborted march leaves copies of force rows in flight
+    if (FORCE == FORCE_ANY) cp_async_wait<0>();
     if (aborted) {
         if (t == 0) {
             for (int it = issued - SLOTS; it < issued; ++it) {
