@@ -181,18 +181,29 @@ static int band_rows(int ny, int target) {
 // about three more for the copies to arrive.
 static int band_work(int rows) { return rows + 11; }
 
-// Longest block when every block takes the next item as it finishes one (items:
-// number of row iterations and how many such items, in order).
-static long long longest_block(const std::vector<std::pair<int, long long>> &items, int blocks) {
-    std::vector<long long> heap(blocks, 0);
-    const auto later = [](long long x, long long y) { return x > y; };
+// Longest block when every block takes the next item as it finishes one.
+// items[r]: how many bands of r rows, longest first.  Blocks with the same load
+// are counted together, which takes a few steps per band height instead of one
+// per item: the active set of a batch changes often while its problems converge.
+static long long longest_block(const std::vector<long long> &items, long long blocks) {
+    typedef std::pair<long long, long long> Load;  // row iterations, blocks that have them
+    std::vector<Load> heap(1, Load(0, blocks));
+    const auto later = [](const Load &x, const Load &y) { return x.first > y.first; };
     long long longest = 0;
-    for (const auto &it : items)
-        for (long long k = 0; k < it.second; ++k) {
+    for (int rows = (int)items.size() - 1; rows > 0; --rows)
+        for (long long left = items[rows]; left > 0;) {
             std::pop_heap(heap.begin(), heap.end(), later);
-            heap.back() += it.first;
-            longest = std::max(longest, heap.back());
+            const Load least = heap.back();
+            const long long m = std::min(left, least.second);
+            const Load more(least.first + band_work(rows), m);
+            longest = std::max(longest, more.first);
+            heap.back() = more;
             std::push_heap(heap.begin(), heap.end(), later);
+            if (least.second > m) {
+                heap.push_back(Load(least.first, least.second - m));
+                std::push_heap(heap.begin(), heap.end(), later);
+            }
+            left -= m;
         }
     return longest;
 }
@@ -219,63 +230,78 @@ static std::vector<int> problem_order(const mdf_batch *b) {
 static void choose_bands(mdf_batch *b) {
     static const int targets[] = {128, 112, 96, 80, 64, 48, 40, 32, 24, 16, 12, 8, 6, 4, 3, 2};
     const int blocks = std::max(1, b->occ) * b->num_sms, W = b->nt - 8;
-    const std::vector<int> order = problem_order(b);
-    std::vector<int> H(b->count, 2);
-    std::vector<std::pair<int, long long>> items;
+    // the active problems by size: rows, strips and how many (sizes repeat)
+    std::vector<std::pair<std::pair<int, int>, int>> sizes;
+    {
+        std::vector<std::pair<int, int>> all;
+        for (int i = 0; i < b->count; ++i)
+            if (b->active[i]) all.push_back(std::make_pair(b->ctx[i]->ny, (b->ctx[i]->nx + W - 1) / W));
+        std::sort(all.begin(), all.end());
+        for (const auto &s : all) {
+            if (sizes.empty() || sizes.back().first != s) sizes.push_back(std::make_pair(s, 0));
+            ++sizes.back().second;
+        }
+    }
+    std::vector<long long> items;
+    int chosen = targets[0];
     double best = -1.0;
     for (const int target : targets) {
         long long n = 0, work = 0;
-        items.clear();
-        for (const int i : order) {
-            const long long strips = (b->ctx[i]->nx + W - 1) / W;
-            const int ny = b->ctx[i]->ny;
-            H[i] = band_rows(ny, target);
-            const int full = ny / H[i], rest = ny % H[i];
-            if (full) items.push_back(std::make_pair(band_work(H[i]), full * strips));
-            if (rest) items.push_back(std::make_pair(band_work(rest), strips));
+        items.assign(targets[0] + 1, 0);
+        for (const auto &s : sizes) {
+            const int ny = s.first.first, H = band_rows(ny, target), full = ny / H, rest = ny % H;
+            const long long strips = (long long)s.first.second * s.second;
+            items[H] += full * strips;
+            if (rest) items[rest] += strips;
             n += (full + (rest ? 1 : 0)) * strips;
-            work += ((long long)full * band_work(H[i]) + (rest ? band_work(rest) : 0)) * strips;
+            work += ((long long)full * band_work(H) + (rest ? band_work(rest) : 0)) * strips;
         }
         // from five items per block on the longest bands are the best
-        if (best < 0) b->H = H;
         if (n > 5ll * blocks || n == 0) break;
-        std::stable_sort(items.begin(), items.end(),
-                         [](const std::pair<int, long long> &x, const std::pair<int, long long> &y) {
-                             return x.first > y.first;
-                         });
         const double cost = 0.8 * (double)work / blocks +
-                            0.2 * (double)longest_block(items, (int)std::min((long long)blocks, n));
+                            0.2 * (double)longest_block(items, std::min((long long)blocks, n));
         if (best < 0 || cost < best) {
             best = cost;
-            b->H = H;
+            chosen = target;
         }
     }
+    for (int i = 0; i < b->count; ++i) b->H[i] = b->active[i] ? band_rows(b->ctx[i]->ny, chosen) : 2;
     b->bands_chosen = true;
 }
 
 // Work items of the active problems, longest first: marches by the rows of the
 // band (their blocks take the next item as they finish one), tiles by problem.
+// A problem has bands of at most two heights, so its bands are sorted as two runs
+// and not one by one.
 static mdf_status build_items(mdf_batch *b) {
-    std::vector<std::pair<int, BatchItem>> items;
+    struct Run {
+        int rows, problem, by0, by1;  // band rows [by0, by1) of a problem
+    };
+    std::vector<Run> runs;
     std::vector<BatchItem> table;
     try {
         if (!b->bands_chosen) choose_bands(b);
-        const int W = b->nt - 8;
+        const int tw = b->tile ? TILE_X : b->nt - 8;
+        size_t n = 0;
         for (const int i : problem_order(b)) {
-            const mdf_ctx *c = b->ctx[i];
-            const int tw = b->tile ? TILE_X : W, th = b->tile ? TILE_Y : b->H[i];
-            const int gx = (c->nx + tw - 1) / tw, gy = (c->ny + th - 1) / th;
-            for (int by = 0; by < gy; ++by) {
-                const int rows = std::min(th, c->ny - by * th);
-                for (int bx = 0; bx < gx; ++bx)
-                    items.push_back(std::make_pair(b->tile ? 0 : rows, BatchItem{i, bx, by, 0}));
+            const int ny = b->ctx[i]->ny, th = b->tile ? TILE_Y : b->H[i];
+            const int full = ny / th, all = (ny + th - 1) / th;
+            if (b->tile) {
+                runs.push_back(Run{0, i, 0, all});
+            } else {
+                if (full) runs.push_back(Run{th, i, 0, full});
+                if (all > full) runs.push_back(Run{ny - full * th, i, full, all});
             }
+            n += (size_t)all * ((b->ctx[i]->nx + tw - 1) / tw);
         }
-        std::stable_sort(items.begin(), items.end(),
-                         [](const std::pair<int, BatchItem> &x, const std::pair<int, BatchItem> &y) {
-                             return x.first > y.first;
-                         });
-        for (const auto &it : items) table.push_back(it.second);
+        if (!b->tile)
+            std::stable_sort(runs.begin(), runs.end(), [](const Run &x, const Run &y) { return x.rows > y.rows; });
+        table.reserve(n);
+        for (const Run &r : runs) {
+            const int gx = (b->ctx[r.problem]->nx + tw - 1) / tw;
+            for (int by = r.by0; by < r.by1; ++by)
+                for (int bx = 0; bx < gx; ++bx) table.push_back(BatchItem{r.problem, bx, by, 0});
+        }
     } catch (const std::bad_alloc &) {
         return bfail(b, MDF_E_NOMEM, "host allocation of the work items failed");
     }
