@@ -292,7 +292,7 @@ long long mdf_steps_done(const mdf_ctx *ctx);
  * the same context (or thread). */
 const char *mdf_last_error(const mdf_ctx *ctx);
 
-/* Launch geometry of the fused step kernel: info[0] threads per block,
+/* Launch geometry of the fused step kernel with the force at hand: info[0] threads per block,
  * info[1] output columns per block, info[2] rows per block, info[3] blocks in
  * x, info[4] blocks in y, info[5] dynamic shared memory bytes,
  * info[6] blocks resident per SM (occupancy query; 0 without a GPU). */
@@ -310,9 +310,11 @@ mdf_status mdf_launch_info(const mdf_ctx *ctx, int info[8]);
  * (every storage mode, not with the alpha = 0 distribution; the only plan
  * for 16-bit storage off the periodic fast path).  mdf_create times every
  * candidate plan for a few steps and keeps the fastest (the tile kernel only
- * if it beats the best march by more than 10 %); this call replaces that
- * choice.  Waits for the context's stream; MDF_E_INVALID for an unsupported
- * block size. */
+ * if it beats the best march by more than 10 %), and the fastest march for a
+ * constant force and for force fields and sources, whose plan is then in use
+ * while such a force is set (the values are the same); this call replaces
+ * those choices.  Waits for the context's stream; MDF_E_INVALID for an
+ * unsupported block size. */
 mdf_status mdf_set_launch(mdf_ctx *ctx, int threads, int rows_per_block);
 
 /* Kernel family of the current launch plan: 0 march, 1 tile (-1 for NULL). */

@@ -183,55 +183,131 @@ static mdf_status wait_stream(mdf_ctx *c, double timeout_s) {
     return check_device_error(c);
 }
 
+struct TuneEvents {
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    ~TuneEvents() {
+        if (e0) cudaEventDestroy(e0);
+        if (e1) cudaEventDestroy(e1);
+    }
+};
+
+// Milliseconds of `launches` steps with plan p and arguments a from buffer 0 into
+// buffer 1.
+static mdf_status time_plan(mdf_ctx *c, const TuneEvents &ev, const StepPlan &p, StepArgs a, int launches, float *ms) {
+    c->plan = p;
+    mdf_status s = encode_maps(c);
+    if (s != MDF_OK) return s;
+    a.W = p.W;
+    a.H = p.H;
+    a.fout = c->buf[1];
+    a.fin = c->buf[0];
+    CK(c, step_launch(&c->tmap[0], a, c->kind, p, 0));
+    CK(c, cudaEventRecord(ev.e0, 0));
+    for (int r = 0; r < launches; ++r) CK(c, step_launch(&c->tmap[0], a, c->kind, p, 0));
+    CK(c, cudaEventRecord(ev.e1, 0));
+    CK(c, cudaEventSynchronize(ev.e1));
+    CK(c, cudaEventElapsedTime(ms, ev.e0, ev.e1));
+    return MDF_OK;
+}
+
 // Launch-plan autotuner: time every candidate plan (march block size and
-// band height, or the tile kernel) for a few steps from the initial state
-// in buffer 0 (which keeps its contents; the output goes to buffer 1) and
-// keep the fastest.  March plans compute the same values whatever the band
+// band height, or the tile kernel) for a few steps and keep the fastest.  March
+// plans compute the same values whatever the band
 // split; the tile kernel is taken only when it beats the best march by more
 // than 10 %, so that timing noise near the crossover cannot flip the kernel
 // (and the last bits of the results) from one run to the next.
+// The steps start from a state in motion, because a power-law fluid at rest skips
+// the viscosity solve (1200 x 700 power-law cavity: at rest 128 threads looked
+// the faster, in motion they take 46.8 us a step against 41.9 of 256).  The
+// marches of the periodic fast path and the wall path have a kernel for each kind
+// of force, so those within a tenth of each other are timed again for each kind
+// (1200 x 700 channel with a source: 35.1 us with the plan of the unforced kernel,
+// 32.6 with its own); the choice between march and tile is that of the unforced
+// kernels.
+// Leaves both buffers overwritten.
 static mdf_status autotune(mdf_ctx *c) {
+    for (StepPlan &p : c->kind_plan) p = c->cand[0];
     if (c->ncand > 1) {
-        cudaEvent_t e0, e1;
-        CK(c, cudaEventCreate(&e0));
-        CK(c, cudaEventCreate(&e1));
-        float best = 1e30f, best_tile = 1e30f;
-        int best_i = 0, tile_i = -1;
-        // two passes over the candidates, 8 timed launches each; keep the
-        // fastest time seen per candidate
-        for (int pass = 0; pass < 2; ++pass)
-        for (int i = 0; i < c->ncand; ++i) {
-            c->plan = c->cand[i];
-            mdf_status s = encode_maps(c);
-            if (s != MDF_OK) return s;
+        const size_t N = (size_t)c->nx * c->ny;
+        mdf_status s = ensure_scratch(c, 3 * N * sizeof(float));
+        if (s != MDF_OK) return s;
+        float *u = c->scratch;
+        CK(c, aux_stir(c->aux, 0.01f * (float)c->prm.c, u, u + N, u + 2 * N, 0));
+        CK(c, aux_init(c->aux, u, u + N, u + 2 * N, c->buf[0], 0));
+        c->plan = c->cand[0];
+        s = encode_maps(c);
+        if (s != MDF_OK) return s;
+        for (int k = 0; k < 2; ++k) {  // the strain rates build up from equilibrium
             StepArgs a = c->args;
             a.W = c->plan.W;
             a.H = c->plan.H;
-            a.fout = c->buf[1];
-            a.fin = c->buf[0];
-            CK(c, step_launch(&c->tmap[0], a, c->kind, c->plan, 0));
-            CK(c, cudaEventRecord(e0, 0));
-            for (int r = 0; r < 8; ++r) CK(c, step_launch(&c->tmap[0], a, c->kind, c->plan, 0));
-            CK(c, cudaEventRecord(e1, 0));
-            CK(c, cudaEventSynchronize(e1));
-            float ms = 0.0f;
-            CK(c, cudaEventElapsedTime(&ms, e0, e1));
-            if (c->plan.kind == PLAN_TILE) {
-                if (ms < best_tile) {
-                    best_tile = ms;
-                    tile_i = i;
-                }
-            } else if (ms < best) {
-                best = ms;
-                best_i = i;
-            }
+            a.fin = c->buf[k];
+            a.fout = c->buf[1 - k];
+            CK(c, step_launch(&c->tmap[k], a, c->kind, c->plan, 0));
         }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        c->plan = c->cand[(tile_i >= 0 && best_tile < 0.9f * best) ? tile_i : best_i];
+        TuneEvents ev;
+        CK(c, cudaEventCreate(&ev.e0));
+        CK(c, cudaEventCreate(&ev.e1));
+        // the fastest time seen of every candidate over two passes; the second
+        // one leaves out those that are far behind their family's best.  Fewer
+        // launches where one takes tens of microseconds and the events resolve it
+        const int launches = N < (1 << 18) ? 6 : 3;
+        float best[mdf_ctx::kMaxCandidates], family[2] = {1e30f, 1e30f};
+        for (int pass = 0; pass < 2; ++pass)
+            for (int i = 0; i < c->ncand; ++i) {
+                const int f = c->cand[i].kind == PLAN_TILE;
+                if (pass == 0) best[i] = 1e30f;
+                else if (best[i] > 1.15f * family[f]) continue;
+                float ms = 0.0f;
+                s = time_plan(c, ev, c->cand[i], c->args, launches, &ms);
+                if (s != MDF_OK) return s;
+                best[i] = fminf(best[i], ms);
+                family[f] = fminf(family[f], ms);
+            }
+        const int tile = family[1] < 0.9f * family[0];
+        for (int i = 0; i < c->ncand; ++i)
+            if ((c->cand[i].kind == PLAN_TILE) == (tile != 0) && best[i] == family[tile])
+                for (StepPlan &p : c->kind_plan) p = c->cand[i];
+        const int walls = c->xwall || c->ywall;
+        const bool kinds = fast_path_applies(c->kind, c->args.power_law, walls) ||
+                           (!c->prm.rho0 && walls_path_applies(c->kind, c->args.power_law, walls, c->prm.storage));
+        for (int kind = FORCE_CONST; !tile && kinds && kind < FORCE_KINDS; ++kind) {
+            // any finite planes do for a force field: those of the state
+            StepArgs a = c->args;
+            a.force_mode = a.force_mode_d = kind == FORCE_CONST ? 1 : 2;
+            a.Fxp = a.Fxdp = c->buf[0];
+            a.Fyp = a.Fydp = c->buf[0] + c->plane;
+            float t[mdf_ctx::kMaxCandidates], least = 1e30f;
+            int rivals = 0;
+            for (int i = 0; i < c->ncand; ++i) {
+                t[i] = 1e30f;
+                rivals += c->cand[i].kind == PLAN_MARCH && best[i] <= 1.1f * family[0];
+            }
+            for (int pass = 0; rivals > 1 && pass < 2; ++pass)
+                for (int i = 0; i < c->ncand; ++i) {
+                    if (c->cand[i].kind != PLAN_MARCH || best[i] > 1.1f * family[0]) continue;
+                    float ms = 0.0f;
+                    s = time_plan(c, ev, c->cand[i], a, launches, &ms);
+                    if (s != MDF_OK) return s;
+                    t[i] = fminf(t[i], ms);
+                    if (t[i] < least) {
+                        least = t[i];
+                        c->kind_plan[kind] = c->cand[i];
+                    }
+                }
+        }
     }
-    c->args.W = c->plan.W;
-    c->args.H = c->plan.H;
+    return MDF_OK;
+}
+
+// The plan of the kind of force at hand (a plan set by mdf_set_launch stays).
+static mdf_status choose_plan(mdf_ctx *c) {
+    if (c->pinned) return MDF_OK;
+    const StepPlan &p = c->kind_plan[force_kind(c->args)];
+    if (p.kind == c->plan.kind && p.NT == c->plan.NT && p.W == c->plan.W && p.H == c->plan.H) return MDF_OK;
+    c->plan = p;
+    c->args.W = p.W;
+    c->args.H = p.H;
     return encode_maps(c);
 }
 
@@ -497,18 +573,19 @@ static mdf_status create_ctx(const mdf_grid *grid, const mdf_fluid *fluid, const
     a.pdw = pack_pair(a.dt * 0.2f);
     CKC(encode_maps(c));
 
+    if (tune) CKC(autotune(c));
+    else
+        for (StepPlan &p : c->kind_plan) p = c->plan;
+    c->plan = c->kind_plan[FORCE_NONE];
+    c->args.W = c->plan.W;
+    c->args.H = c->plan.H;
+    CKC(encode_maps(c));
     // Rest state.
     CKE(ensure_scratch(c, 3 * N * sizeof(float)) == MDF_OK ? cudaSuccess : cudaErrorMemoryAllocation);
     CKE(cudaMemset(c->scratch, 0, 3 * N * sizeof(float)));
     CKE(aux_init(x, c->scratch, c->scratch + N, c->scratch + 2 * N, c->buf[0], 0));
     CKE(aux_snapshot(x, c->buf[0], c->snap_u, c->snap_v, 0));
     CKE(cudaDeviceSynchronize());
-    if (tune) CKC(autotune(c));
-    else {
-        c->args.W = c->plan.W;
-        c->args.H = c->plan.H;
-        CKC(encode_maps(c));
-    }
     c->cur = 0;
     *out = c;
     return MDF_OK;
@@ -572,7 +649,7 @@ static mdf_status update_force_d(mdf_ctx *c) {
         a.Fydp = c->Fydp;
     }
     ++c->args_version;
-    return MDF_OK;
+    return choose_plan(c);
 }
 
 mdf_status mdf_set_force(mdf_ctx *c, int mode, double fx, double fy, const float *Fx, const float *Fy,
@@ -653,7 +730,7 @@ mdf_status mdf_set_source(mdf_ctx *c, int mode, double r, const float *R, int on
     c->aux.Rc = a.Rc;
     c->aux.Rp = a.Rp;
     ++c->args_version;
-    return MDF_OK;
+    return choose_plan(c);
 }
 
 mdf_status mdf_set_metrics(mdf_ctx *c, const double *xi_x, const double *xi_y, const double *eta_x,
@@ -1093,6 +1170,7 @@ mdf_status mdf_set_launch(mdf_ctx *c, int threads, int rows_per_block) {
     CK(c, cudaStreamSynchronize(c->stream));
     if (c->cstream) CK(c, cudaStreamSynchronize(c->cstream));
     c->plan = p;
+    c->pinned = true;
     c->args.W = p.W;
     c->args.H = p.H;
     drop_graphs(c);

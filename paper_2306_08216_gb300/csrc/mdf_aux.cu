@@ -164,6 +164,20 @@ __global__ void init_kernel(AuxArgs a, const float *u, const float *v, const flo
     }
 }
 
+// Velocities that differ from node to node without a pattern.
+__global__ void stir_kernel(int nx, float amp, float *u, float *v, float *p) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+    if (x >= nx) return;
+    const long long n = (long long)y * nx + x;
+    unsigned h = (unsigned)x * 2654435761u + (unsigned)y * 40503u;
+    h ^= h >> 15;
+    h *= 2246822519u;
+    h ^= h >> 13;
+    u[n] = amp * ((float)(h & 0xffff) * (1.0f / 32768.0f) - 1.0f);
+    v[n] = amp * ((float)(h >> 16) * (1.0f / 32768.0f) - 1.0f);
+    p[n] = 0.0f;
+}
+
 // alpha = 0 distribution at equilibrium with the given rho_0 and the
 // velocity of the current alpha = 1, 2 state (FP32 storage).
 __global__ void init_rho0_kernel(AuxArgs a, const float *rho0, float *f) {
@@ -607,6 +621,11 @@ static void pack_planes(const AuxArgs &a, const float *f, float *dense, cudaStre
         pack_kernel<4, K><<<rows_grid(a.nx, a.ny, 512), 128, 0, st>>>(a, f, dense);
     else
         pack_kernel<1, K><<<rows_grid(a.nx, a.ny, 128), 128, 0, st>>>(a, f, dense);
+}
+
+cudaError_t aux_stir(const AuxArgs &a, float amp, float *u, float *v, float *p, cudaStream_t st) {
+    stir_kernel<<<rows_grid(a.nx, a.ny, 128), 128, 0, st>>>(a.nx, amp, u, v, p);
+    return cudaGetLastError();
 }
 
 cudaError_t aux_pack(const AuxArgs &a, const float *f, float *dense, cudaStream_t st) {

@@ -28,6 +28,8 @@ struct FieldPtrs {
 };
 
 cudaError_t aux_init(const AuxArgs &a, const float *u, const float *v, const float *p, float *f, cudaStream_t st);
+// A field in motion everywhere (velocities of +- amp, zero pressure), dense.
+cudaError_t aux_stir(const AuxArgs &a, float amp, float *u, float *v, float *p, cudaStream_t st);
 cudaError_t aux_pack(const AuxArgs &a, const float *f, float *dense, cudaStream_t st);
 cudaError_t aux_unpack(const AuxArgs &a, const float *dense, float *f, cudaStream_t st);
 cudaError_t aux_pad_field(const AuxArgs &a, const float *src, float *dst, cudaStream_t st);

@@ -59,6 +59,9 @@ struct mdf_ctx {
     mdf::StepPlan cand[kMaxCandidates];
     int ncand = 0;
     mdf::StepPlan plan{};
+    // the tuned plan of each kind of force; mdf_set_launch replaces them for good
+    mdf::StepPlan kind_plan[mdf::FORCE_KINDS];
+    bool pinned = false;
     mdf::StepArgs args{};
     mdf::AuxArgs aux{};
     cudaStream_t stream = nullptr;

@@ -127,16 +127,6 @@ __device__ __forceinline__ void tma_load_row(const CUtensorMap *map, uint64_t *b
         : "memory");
 }
 
-// What of body force and source a march kernel is compiled for: FORCE_ANY reads
-// the modes at run time and keeps a ring of force field rows; the constant force
-// needs neither the ring nor its copies and waits, and keeps the TMA slots of the
-// unforced kernel (channel of 1200 x 700 nodes: 35.1 -> 30.2 us a step).
-constexpr int FORCE_NONE = 0, FORCE_CONST = 1, FORCE_ANY = 2;
-inline int force_kind(const StepArgs &a) {
-    if (!a.force_mode && !a.force_mode_d && !a.r_mode) return FORCE_NONE;
-    return a.force_mode <= 1 && a.force_mode_d <= 1 && !a.r_mode ? FORCE_CONST : FORCE_ANY;
-}
-
 // Four bytes from global to shared memory, asynchronously.
 __device__ __forceinline__ void cp_async4(void *dst, const float *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
