@@ -213,7 +213,7 @@ cudaError_t rho0_launch(const CUtensorMap *tmap, const StepArgs &args, int metri
 // distribution with FP32 storage.  It is also the only kernel for 16-bit
 // storage outside the periodic fast path.
 bool tile_path_applies(int storage, int rho0);
-cudaError_t tile_occupancy(int metric, int power_law, int walls, int storage, int rho0, int *tx, int *ty, int *occ,
+cudaError_t tile_occupancy(int metric, int power_law, int walls, int storage, int rho0, int ts, int *occ,
                            int *smem);
 cudaError_t tile_launch(const StepArgs &args, int metric, const StepPlan &plan, cudaStream_t stream);
 // The same kernel over the work items (problem, tile x, tile y) of a batch.

@@ -93,33 +93,23 @@ int step_candidates(int metric, int power_law, int walls, int storage, int rho0,
         for (int waves = 1; waves <= 2 && n < max; ++waves) fill_plan(nts[i], occ, smem, waves, nx, ny, num_sms, &out[n++]);
     }
     // the tile kernel, last: the marches stay the default
-    if (tile_path_applies(storage, rho0) && n < max) {
-        int tx = 0, ty = 0, occ = 0, smem = 0;
-        const cudaError_t e = tile_occupancy(metric, power_law, walls, storage, rho0, &tx, &ty, &occ, &smem);
-        if (e != cudaSuccess) {
-            *err = e;
-            return n;
-        }
-        if (occ >= 1) {
-            const auto tile_plan = [&](int tw, int th) {
-                StepPlan &p = out[n++];
-                p.kind = PLAN_TILE;
-                p.NT = tile_threads(tw, storage, rho0 != 0);
-                p.W = tw;
-                p.H = th;
-                p.gx = (nx + tw - 1) / tw;
-                p.gy = (ny + th - 1) / th;
-                p.smem = smem;
-                p.occ = occ;
-            };
-            tile_plan(tx, ty);
-            // 8 x 8 tiles while a grid of them still fits the SMs at three
-            // blocks each: from about there on their larger halo costs more than
-            // the shorter phases give
-            const long long small = (long long)((nx + 7) / 8) * ((ny + 7) / 8);
-            if (storage == STORAGE_FP32 && !rho0 && n < max && small <= 3ll * (num_sms > 0 ? num_sms : 1))
-                tile_plan(kSmallTile, kSmallTile);
-        }
+    if (!tile_path_applies(storage, rho0)) return n;
+    // 8 x 8 tiles while a grid of them still fits the SMs at three
+    // blocks each: from about there on their larger halo costs more than
+    // the shorter phases give
+    const long long small = (long long)((nx + 7) / 8) * ((ny + 7) / 8);
+    const bool small_too = storage == STORAGE_FP32 && !rho0 && small <= 3ll * (num_sms > 0 ? num_sms : 1);
+    for (const int ts : {TILE_X, kSmallTile}) {
+        if (n >= max || (ts == kSmallTile && !small_too)) break;
+        StepPlan &p = out[n];
+        *err = tile_occupancy(metric, power_law, walls, storage, rho0, ts, &p.occ, &p.smem);
+        if (*err != cudaSuccess || p.occ < 1) break;
+        p.kind = PLAN_TILE;
+        p.NT = tile_threads(ts, storage, rho0 != 0);
+        p.W = p.H = ts;
+        p.gx = (nx + ts - 1) / ts;
+        p.gy = (ny + ts - 1) / ts;
+        ++n;
     }
     return n;
 }

@@ -9,15 +9,13 @@ MDF_TILE_DEFINE(STORAGE_FP32)
 // Every storage mode; the alpha = 0 distribution with FP32 storage.
 bool tile_path_applies(int storage, int rho0) { return !rho0 || storage == STORAGE_FP32; }
 
-cudaError_t tile_occupancy(int metric, int power_law, int walls, int storage, int rho0, int *tx, int *ty, int *occ,
+cudaError_t tile_occupancy(int metric, int power_law, int walls, int storage, int rho0, int ts, int *occ,
                            int *smem) {
-    *tx = kTX;
-    *ty = kTY;
-    if (rho0) return tile_occupancy_rho0(metric, power_law, walls, occ, smem);
+    if (rho0) return tile_occupancy_rho0(metric, power_law, walls, ts, occ, smem);
     switch (storage) {
-        case STORAGE_FP16: return tile_occupancy_st<STORAGE_FP16>(metric, power_law, walls, occ, smem);
-        case STORAGE_BF16: return tile_occupancy_st<STORAGE_BF16>(metric, power_law, walls, occ, smem);
-        default: return tile_occupancy_st<STORAGE_FP32>(metric, power_law, walls, occ, smem);
+        case STORAGE_FP16: return tile_occupancy_st<STORAGE_FP16>(metric, power_law, walls, ts, occ, smem);
+        case STORAGE_BF16: return tile_occupancy_st<STORAGE_BF16>(metric, power_law, walls, ts, occ, smem);
+        default: return tile_occupancy_st<STORAGE_FP32>(metric, power_law, walls, ts, occ, smem);
     }
 }
 

@@ -8,8 +8,8 @@
 
 namespace mdf {
 
-cudaError_t tile_occupancy_rho0(int metric, int power_law, int walls, int *occ, int *smem) {
-    MDF_TILE_DISPATCH_RHO0(tile_occupancy_t, occ, smem)
+cudaError_t tile_occupancy_rho0(int metric, int power_law, int walls, int ts, int *occ, int *smem) {
+    MDF_TILE_DISPATCH_RHO0(tile_occupancy_t, ts, occ, smem)
 }
 
 cudaError_t tile_launch_rho0(const StepArgs &args, int metric, const StepPlan &plan, cudaStream_t stream) {

@@ -551,13 +551,23 @@ constexpr int tile_smem() {
     return T::B_BYTES + T::F_BYTES + (PL ? T::K_BYTES : 0) + (RHO0 ? T::B0_BYTES + T::F0_BYTES : 0);
 }
 
-template <int MK, bool PL, bool WALLS, int ST, bool RHO0 = false>
-cudaError_t tile_occupancy_t(int *occ, int *smem) {
-    auto k = tile_kernel<kTX, kTY, MK, PL, WALLS, ST, RHO0>;
-    *smem = tile_smem<MK, PL, WALLS, RHO0>();
+template <int MK, bool PL, bool WALLS, int ST, bool RHO0, int TS>
+cudaError_t tile_occupancy_ts(int *occ, int *smem) {
+    auto k = tile_kernel<TS, TS, MK, PL, WALLS, ST, RHO0>;
+    *smem = tile_smem<MK, PL, WALLS, RHO0, TS>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, tile_threads(kTX, ST, RHO0), *smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, tile_threads(TS, ST, RHO0), *smem);
+}
+
+// ts: side of the tile, kTX or (FP32 storage without the alpha = 0 lane) kSmallTile.
+template <int MK, bool PL, bool WALLS, int ST, bool RHO0 = false>
+cudaError_t tile_occupancy_t(int ts, int *occ, int *smem) {
+    if constexpr (ST == STORAGE_FP32 && !RHO0) {
+        if (ts == kSmallTile) return tile_occupancy_ts<MK, PL, WALLS, ST, RHO0, kSmallTile>(occ, smem);
+    }
+    if (ts != kTX) return cudaErrorInvalidConfiguration;
+    return tile_occupancy_ts<MK, PL, WALLS, ST, RHO0, kTX>(occ, smem);
 }
 
 // One step with tiles of TS x TS nodes.
@@ -658,13 +668,13 @@ cudaError_t tile_batch_launch_t(const BatchItem *items, int nitems, const StepAr
 }  // namespace
 
 // The tile kernel with the alpha = 0 lane (mdf_step_tile_rho0.cu).
-cudaError_t tile_occupancy_rho0(int metric, int power_law, int walls, int *occ, int *smem);
+cudaError_t tile_occupancy_rho0(int metric, int power_law, int walls, int ts, int *occ, int *smem);
 cudaError_t tile_launch_rho0(const StepArgs &args, int metric, const StepPlan &plan, cudaStream_t stream);
 
 // The tile kernel's launch helpers for one storage mode ST (defined in
 // mdf_step_tile.cu for FP32 and mdf_step_tile16.cu for FP16 and BF16).
 template <int ST>
-cudaError_t tile_occupancy_st(int metric, int power_law, int walls, int *occ, int *smem);
+cudaError_t tile_occupancy_st(int metric, int power_law, int walls, int ts, int *occ, int *smem);
 template <int ST>
 cudaError_t tile_launch_st(const StepArgs &args, int metric, const StepPlan &plan, cudaStream_t stream);
 template <int ST>
@@ -676,8 +686,8 @@ cudaError_t tile_batch_launch_st(const BatchItem *items, int nitems, const StepA
 // Definitions of the four helpers for storage mode ST in the including file.
 #define MDF_TILE_DEFINE(ST)                                                                                        \
     template <>                                                                                                    \
-    cudaError_t tile_occupancy_st<ST>(int metric, int power_law, int walls, int *occ, int *smem) {                 \
-        MDF_TILE_DISPATCH(ST, tile_occupancy_t, occ, smem)                                                         \
+    cudaError_t tile_occupancy_st<ST>(int metric, int power_law, int walls, int ts, int *occ, int *smem) {         \
+        MDF_TILE_DISPATCH(ST, tile_occupancy_t, ts, occ, smem)                                                     \
     }                                                                                                              \
     template <>                                                                                                    \
     cudaError_t tile_launch_st<ST>(const StepArgs &args, int metric, const StepPlan &plan, cudaStream_t stream) {  \
