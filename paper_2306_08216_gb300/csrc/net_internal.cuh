@@ -103,7 +103,6 @@ struct BiasArgs {
 cudaError_t bias_grads(BiasArgs a, cudaStream_t st);
 
 // Elementwise / layout kernels (n = element count unless stated).
-cudaError_t silu_forward(const bf16 *z, bf16 *y, long long n, cudaStream_t st);
 cudaError_t pool_forward(const bf16 *x, bf16 *y, int B, int R, int C, cudaStream_t st);    // R = input side
 // dz [B][R][R][C] = silu'(z) (dy [B][R/2][R/2][C] / 4 + skip), the gradient
 // through a pooled activation that also feeds a skip connection; the quarter

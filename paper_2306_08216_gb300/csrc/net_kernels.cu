@@ -298,11 +298,6 @@ __global__ void __launch_bounds__(128) bias_grad_kernel(const BiasArgs a) {
 
 // ------------------------------------------------------------- elementwise
 
-__global__ void silu_fwd_kernel(const bf16 *z, bf16 *y, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        y[i] = silu_bf16(z[i]);
-}
-
 // The elementwise kernels below move 8 BF16 channels (16 bytes) per thread
 // and step: C is a multiple of 32, so a group never straddles two pixels.
 typedef uint4 bf16x8;
@@ -550,10 +545,6 @@ cudaError_t bias_grads(BiasArgs a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t silu_forward(const bf16 *z, bf16 *y, long long n, cudaStream_t st) {
-    silu_fwd_kernel<<<blocks_for(n), 256, 0, st>>>(z, y, n);
-    return cudaGetLastError();
-}
 cudaError_t pool_forward(const bf16 *x, bf16 *y, int B, int R, int C, cudaStream_t st) {
     if (C % 8) return cudaErrorInvalidValue;
     pool_fwd_kernel<<<blocks_for((long long)B * R * R * C / 32), 256, 0, st>>>(
