@@ -387,9 +387,8 @@ mdf_status mdf_batch_info(const mdf_batch *batch, long long info[6]);
 /* Kernel of the batch step: 0 marches (work items are strips x bands of
  * each problem), 1 tiles (work items are the 16 x 16 tiles of each
  * problem, the tile kernel of mdf_set_launch), 2 marches in rolled form
- * (uniform and separable grids: the same values as 0 from a body a fifth
- * the size, faster on a full GPU, slower on a few small problems; the only
- * march form with 16-bit storage).
+ * (uniform and separable grids: the same values as 0 in nearly the same
+ * time; the only march form with 16-bit storage).
  * mdf_batch_create times them and keeps the faster march unless the tiles
  * are more than 10 % faster, and mdf_batch_set_active times them again over
  * the problems that remain (FP32 batches); mdf_batch_set_launch fixes the

@@ -4,10 +4,11 @@
 // buffers, metrics, forcing and residual snapshot), so every single-problem
 // call (mdf_fields, mdf_get_distributions, mdf_residual, ...) works on it.
 // mdf_batch_step advances all of them together: one launch per time step of
-// a persistent kernel whose blocks walk a table of work items ordered
-// largest problem first, with the problems' arguments (and TMA descriptors)
+// a persistent kernel whose blocks walk a table of work items, with the
+// problems' arguments (and TMA descriptors)
 // in global memory: either marches (problem, strip, band: walls_batch_kernel
-// or batch_kernel) or tiles (problem, tile x, tile y: tile_batch_kernel).
+// or batch_kernel; longest bands first) or tiles (problem, tile x, tile y:
+// tile_batch_kernel; largest problem first).
 // The batch times both at creation and keeps the faster.  Repeated steps are
 // replayed from captured CUDA graphs of kGraphSteps launches.
 #include <math.h>
@@ -41,7 +42,7 @@ struct mdf_batch {
     int nitems = 0, grid = 0, occ = 0, smem = 0;
     bool bands_chosen = false;                     // H holds the band heights of the active set
     int tile = 0, occ_tile = 0, smem_tile = 0;     // tile mode: one work item per 16 x 16 tile
-    int roll = 0;                                  // march mode: the rolled register-window march
+    int roll = 0;                                  // march mode: its loop not unrolled
     int pinned = 0;                                // mode set by mdf_batch_set_launch (no re-timing)
     int storage = 0;                               // StorageKind of every problem (16-bit: tile mode only)
     int forced = 0;                                // some problem has a force, force rate or source
@@ -325,10 +326,8 @@ static mdf_status build_items(mdf_batch *b) {
 
 // Time a few steps of each kernel over the active problems (their current
 // buffers are read and the other ones written, so the states are unchanged;
-// the batch's streams must be idle): the register-window march unrolled or
-// rolled (the same values; the faster is kept: the rolled one wins on a
-// full GPU, where the unrolled body misses the instruction cache, the
-// unrolled one on a few small problems, where row latency decides), and
+// the batch's streams must be idle): the march with its loop unrolled by two or
+// rolled (the same values; within 1.5 % of each other, see march_walls), and
 // the tile kernel, kept only when more than 10 % faster than the better
 // march (its last bits differ).  Run at creation and whenever the active
 // set changes: a batch whose remaining problems are few and small steps

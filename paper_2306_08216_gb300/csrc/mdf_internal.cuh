@@ -179,14 +179,14 @@ struct BatchItem {
     int problem, bx, by, pad;
 };
 // storage: the batch's storage mode (16-bit: uniform and separable grids
-// only, rolled form).  roll: the rolled form of the register-window march
-// (uniform and separable grids; ignored on curvilinear grids).
+// only, rolled form).  roll: the march loop not unrolled (uniform and separable
+// grids; ignored on curvilinear grids).
 cudaError_t batch_occupancy(int metric, int power_law, int walls, int storage, int *nt, int *occ, int *smem);
 cudaError_t batch_launch(const BatchItem *items, int nitems, int *queue, const StepArgs *args, const CUtensorMap *maps, int metric,
                          int power_law, int walls, int grid, int forced, int roll, int storage, cudaStream_t stream);
 
-// Walls and/or power law on uniform/separable grids, FP32 storage, in the
-// register-window form of the fast path (mdf_step_walls.cu).
+// Walls and/or power law on uniform/separable grids, FP32 storage, marched
+// like the fast path (mdf_step_walls.cu).
 bool walls_path_applies(int metric, int power_law, int walls, int storage);
 cudaError_t walls_occupancy(int metric, int power_law, int nt, int *occ, int *smem);
 cudaError_t walls_launch(const CUtensorMap *tmap, const StepArgs &args, int metric, const StepPlan &plan,

@@ -5,8 +5,8 @@
 // Same time step as the marches (Sec. 2.2 Steps (1)-(4) of arXiv:2306.08216
 // with Eqs. 2.3.24-2.3.25, f32x2 pairs for alpha = u, v, every grid kind,
 // walls by non-equilibrium extrapolation, power law), organised per 2-D
-// tile instead of per band: a block of TX x TY threads owns a TX x TY tile
-// of output nodes and performs the step in three phases separated by
+// tile instead of per band: a block (tile_threads, mdf_internal.cuh) owns a
+// TX x TY tile of output nodes and performs the step in three phases separated by
 // barriers:
 //   A  fhat(t) of the tile plus a halo of 4 (read from L2/HBM with plain
 //      loads) -> fbar^+ of every node of that region into shared memory;
@@ -21,7 +21,7 @@
 // The halo is recomputed (a 16 x 16 tile computes fbar^+ on 24 x 24 nodes
 // and f on 20 x 20), which the marches avoid; in exchange a step is three
 // short phases per block instead of a march of H + 9 rows, and a 257^2 grid
-// is 289 blocks of 8 warps instead of a few hundred 4-warp marches, so
+// is 289 blocks of 9 warps instead of a few hundred 4-warp marches, so
 // small grids are no longer bound by the length of a serial march.
 #pragma once
 
@@ -33,8 +33,9 @@ namespace {
 
 using namespace dev;
 
-// Three 256-thread blocks per SM (at most 85 registers; a few variants spill
-// 20-24 bytes): on the 513^2 trapezoid cavities 18 % faster than two.
+// Three blocks per SM (at most 72 registers of 288 threads, 80 of 256; no FP32 step
+// kernel spills, one batch form 28 bytes, two of the 16-bit batches and two with the
+// alpha = 0 lane 4 to 16): on the 513^2 trapezoid cavities 18 % faster than two.
 constexpr int kTileMinBlocks = 3;
 
 __device__ __forceinline__ F2 pair_of_bits(unsigned long long bits) {

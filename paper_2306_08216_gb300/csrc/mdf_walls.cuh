@@ -1,11 +1,13 @@
 // mdf_walls.cuh -- fused MDF-FDLBM step with non-equilibrium
 // extrapolation walls and/or a power-law fluid, on uniform or separable
-// grids, in the register-window form of the periodic fast path.
+// grids, marched by rows like the periodic fast path.
 //
 // The time step is that of mdf_step.cu (Sec. 2.2 Steps (1)-(4) of
 // arXiv:2306.08216 with Eqs. 2.3.24-2.3.25, f32x2 pairs for alpha = u, v)
 // with the same row march as mdf_step_fast.cu: populations 2 and 4 keep
-// their five-row windows of fbar^+ and f(t+h) in registers, populations 1
+// what their y stencils need of fbar^+ and f(t+h) in registers (five-row windows
+// in march_window, for a single problem; carried sums in march_walls, for
+// batches), populations 1
 // and 3 run their x stencils through double-buffered exchange rows, fhat^+
 // waits in a shared ring, and one barrier orders each row.  On top of that:
 //  * walls (Secs. 4.3-4.4): wall nodes take the non-equilibrium
@@ -21,7 +23,7 @@
 // f(t+h) of a wall node is needed only by the stencils of interior nodes:
 // pops 1 and 3 of a wall column go to the exchange row (written by the
 // thread of the adjacent interior column), pops 2 and 4 of a wall row to the
-// register window of the same column (south: when row 1 is formed; north:
+// registers of the same column (south: when row 1 is formed; north:
 // from row ny-2 through a one-row shared buffer, one iteration later).
 //
 // This header holds the march and its kernel templates; mdf_step_walls.cu
@@ -91,11 +93,13 @@ __device__ __forceinline__ void store_node_st(const StepArgs &a, int row, int X,
 // One block's march over strip bx, band by.  FORCED: body force, force rate
 // or source present (read at run time); otherwise those terms are compiled out.
 // ROLL: the march loop is not unrolled; otherwise it is unrolled by two.  The
-// two compute the same values.  The y stencils carry seven values per stage
+// two compute the same values, in nearly the same time (power-law cavities of
+// 65^2 to 513^2, us a step, unrolled / rolled: 16 of them 75.0 / 75.3, 512
+// 1425 / 1429; Newtonian ones 53.8 / 53.1 and 1175 / 1159).  The y stencils carry seven values per stage
 // from row to row (YCarry): with five-row register windows the loop was either
 // five bodies long, which missed the instruction cache, or rotated a hundred
 // registers a row, and took 168 registers (four blocks of 96 threads per SM;
-// now five).
+// now at most 128 and five).
 // ST: the storage mode of the state (16-bit: fhat is rebuilt from the
 // stored u, v, P and non-equilibrium pairs on load, and stored back in that
 // form, as on the periodic fast path).
@@ -796,8 +800,10 @@ __device__ __forceinline__ void march_window(const CUtensorMap *tmap, const Step
 }
 
 // Resident blocks the register budget is sized for: march_walls 5 x 96 threads
-// (136 registers), march_window 3 x 128 (168: it does not fit 128 without
-// spilling) or 2 x 256.
+// (it takes up to 128 registers; power law on stretched grids spills 8 to 36
+// bytes), march_window 3 x 128 (up to 166) or 2 x 256 (128, spilling 16 to 112
+// bytes except in the plainest forms, and still the faster of the two where its
+// bands fit the grid better: 1200 x 700 power-law cavity 41.8 us a step against 46.8).
 constexpr int kWallsBatchBlocks = 5;
 template <int NT>
 constexpr int walls_min_blocks() {

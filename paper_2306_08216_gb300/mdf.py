@@ -450,7 +450,9 @@ class Solver:
 
     def set_launch(self, threads, rows_per_block=0):
         """threads 128 / 256: a march plan with that block size and band
-        height; threads 0: the 16 x 16 tile kernel."""
+        height; threads 0: the tile kernel, with tiles of 8 x 8 nodes for
+        rows_per_block 8 where the grid is small enough to have them, else of
+        16 x 16.  Replaces the plans the solver chose for every kind of force."""
         _check(lib().mdf_set_launch(self._h, int(threads), int(rows_per_block)), self._h)
 
     def bytes_per_node(self):
