@@ -212,18 +212,18 @@ static mdf_status time_plan(mdf_ctx *c, const TuneEvents &ev, const StepPlan &p,
 
 // Launch-plan autotuner: time every candidate plan (march block size and
 // band height, or the tile kernel) for a few steps and keep the fastest.  March
-// plans compute the same values whatever the band
-// split; the tile kernel is taken only when it beats the best march by more
-// than 10 %, so that timing noise near the crossover cannot flip the kernel
-// (and the last bits of the results) from one run to the next.
+// plans compute the same values whatever the band split; the tile kernel is taken
+// only when it beats the best march by more than 10 %, so that timing noise near
+// the crossover cannot flip the kernel (and the last bits of the results) from one
+// run to the next.
 // The steps start from a state in motion, because a power-law fluid at rest skips
 // the viscosity solve (1200 x 700 power-law cavity: at rest 128 threads looked
 // the faster, in motion they take 46.8 us a step against 41.9 of 256).  The
 // marches of the periodic fast path and the wall path have a kernel for each kind
-// of force, so those within a tenth of each other are timed again for each kind
-// (1200 x 700 channel with a source: 35.1 us with the plan of the unforced kernel,
-// 32.6 with its own); the choice between march and tile is that of the unforced
-// kernels.
+// of force, so the better plans of the two block sizes are timed again for each
+// kind where they are within a tenth of each other (1200 x 700 channel with a
+// source: 35.1 us with the plan of the unforced kernel, 32.6 with its own); the
+// choice between march and tile is that of the unforced kernels.
 // Leaves both buffers overwritten.
 static mdf_status autotune(mdf_ctx *c) {
     for (StepPlan &p : c->kind_plan) p = c->cand[0];
@@ -249,15 +249,17 @@ static mdf_status autotune(mdf_ctx *c) {
         CK(c, cudaEventCreate(&ev.e0));
         CK(c, cudaEventCreate(&ev.e1));
         // the fastest time seen of every candidate over two passes; the second
-        // one leaves out those that are far behind their family's best.  Fewer
-        // launches where one takes tens of microseconds and the events resolve it
-        const int launches = N < (1 << 18) ? 6 : 3;
+        // one leaves out those that cannot win any more.  Fewer launches where one
+        // takes tens of microseconds and the events resolve it
+        const bool small = N < (1 << 18);
+        const int launches = small ? 6 : N < (1 << 22) ? 3 : 2;
+        const float near = small ? 1.15f : 1.05f;
         float best[mdf_ctx::kMaxCandidates], family[2] = {1e30f, 1e30f};
         for (int pass = 0; pass < 2; ++pass)
             for (int i = 0; i < c->ncand; ++i) {
                 const int f = c->cand[i].kind == PLAN_TILE;
                 if (pass == 0) best[i] = 1e30f;
-                else if (best[i] > 1.15f * family[f]) continue;
+                else if (best[i] > near * family[f] || (f && best[i] > near * family[0])) continue;
                 float ms = 0.0f;
                 s = time_plan(c, ev, c->cand[i], c->args, launches, &ms);
                 if (s != MDF_OK) return s;
@@ -265,36 +267,32 @@ static mdf_status autotune(mdf_ctx *c) {
                 family[f] = fminf(family[f], ms);
             }
         const int tile = family[1] < 0.9f * family[0];
+        int chosen = 0, rival = -1;  // the fastest plan; the fastest march of the other block size
         for (int i = 0; i < c->ncand; ++i)
-            if ((c->cand[i].kind == PLAN_TILE) == (tile != 0) && best[i] == family[tile])
-                for (StepPlan &p : c->kind_plan) p = c->cand[i];
+            if (best[i] == family[tile] && (c->cand[i].kind == PLAN_TILE) == (tile != 0)) chosen = i;
+        for (int i = 0; i < c->ncand; ++i)
+            if (c->cand[i].kind == PLAN_MARCH && c->cand[i].NT != c->cand[chosen].NT &&
+                best[i] < 1.1f * family[0] && (rival < 0 || best[i] < best[rival]))
+                rival = i;
+        for (StepPlan &p : c->kind_plan) p = c->cand[chosen];
         const int walls = c->xwall || c->ywall;
         const bool kinds = fast_path_applies(c->kind, c->args.power_law, walls) ||
                            (!c->prm.rho0 && walls_path_applies(c->kind, c->args.power_law, walls, c->prm.storage));
-        for (int kind = FORCE_CONST; !tile && kinds && kind < FORCE_KINDS; ++kind) {
+        for (int kind = FORCE_CONST; !tile && rival >= 0 && kinds && kind < FORCE_KINDS; ++kind) {
             // any finite planes do for a force field: those of the state
             StepArgs a = c->args;
             a.force_mode = a.force_mode_d = kind == FORCE_CONST ? 1 : 2;
             a.Fxp = a.Fxdp = c->buf[0];
             a.Fyp = a.Fydp = c->buf[0] + c->plane;
-            float t[mdf_ctx::kMaxCandidates], least = 1e30f;
-            int rivals = 0;
-            for (int i = 0; i < c->ncand; ++i) {
-                t[i] = 1e30f;
-                rivals += c->cand[i].kind == PLAN_MARCH && best[i] <= 1.1f * family[0];
-            }
-            for (int pass = 0; rivals > 1 && pass < 2; ++pass)
-                for (int i = 0; i < c->ncand; ++i) {
-                    if (c->cand[i].kind != PLAN_MARCH || best[i] > 1.1f * family[0]) continue;
+            float t[2] = {1e30f, 1e30f};
+            for (int pass = 0; pass < 2; ++pass)
+                for (int k = 0; k < 2; ++k) {
                     float ms = 0.0f;
-                    s = time_plan(c, ev, c->cand[i], a, launches, &ms);
+                    s = time_plan(c, ev, c->cand[k ? rival : chosen], a, launches, &ms);
                     if (s != MDF_OK) return s;
-                    t[i] = fminf(t[i], ms);
-                    if (t[i] < least) {
-                        least = t[i];
-                        c->kind_plan[kind] = c->cand[i];
-                    }
+                    t[k] = fminf(t[k], ms);
                 }
+            if (t[1] < t[0]) c->kind_plan[kind] = c->cand[rival];
         }
     }
     return MDF_OK;
