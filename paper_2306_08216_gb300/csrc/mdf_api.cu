@@ -251,9 +251,8 @@ static mdf_status autotune(mdf_ctx *c) {
         // the fastest time seen of every candidate over two passes; the second
         // one leaves out those that cannot win any more.  Fewer launches where one
         // takes tens of microseconds and the events resolve it
-        const bool small = N < (1 << 18);
-        const int launches = small ? 6 : N < (1 << 22) ? 3 : 2;
-        const float near = small ? 1.15f : 1.05f;
+        const int launches = N < (1 << 18) ? 6 : N < (1 << 22) ? 3 : 2;
+        const float near = 1.15f;
         float best[mdf_ctx::kMaxCandidates], family[2] = {1e30f, 1e30f};
         for (int pass = 0; pass < 2; ++pass)
             for (int i = 0; i < c->ncand; ++i) {
